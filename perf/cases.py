@@ -31,7 +31,7 @@ def _case(name, kind, packets, q, routers=1, log2_eta=11, r=5, delta=5, k=60, th
 def listed():
     return [
         # the smallest slots: a campus link's few hundred pairs, where launches and latency count
-        _case("slot_tiny", "slot", 160, 9, log2_eta=6, delta=8, k=3, theta=40, planted=4, lo=45, hi=70, sync=True),
+        _case("slot_tiny", "slot", 160, 9, log2_eta=6, delta=8, k=3, theta=40, planted=4, lo=45, hi=70, slots=3, sync=True),
         # the paper's own dimensions (Sec. 5), one router, the README's loop: the list on the host each slot
         _case("slot_paper", "slot", 1 << 18, 14, delta=6, k=4, lo=2000, hi=8000, slots=4, sync=True),
         # one core-link router at 40 Gb/s, lists left on the device (the pipelined form)
