@@ -128,7 +128,19 @@ struct Clock {
   uint32_t klim2;   // length of the window's 16-bit range, both halves
   uint32_t xe2;     // the stamp whose distance reaches 65535 at the advance, both halves
   uint32_t wrap;    // kNever lies in the 16-bit range of the window
+  // operands of the fused tests (out2, least2), both halves:
+  uint32_t neg_lo2;    // -lo
+  uint32_t top2;       // klim - 1
+  uint32_t neg_top2;   // 1 - klim
+  uint32_t neg_xe2;    // -xe
 };
+__host__ __device__ __forceinline__ uint32_t both(uint32_t v) { return (v & 0xFFFFu) * 0x00010001u; }
+__host__ __device__ __forceinline__ void fused_operands(Clock& c) {
+  c.neg_lo2 = both(0u - c.lo2);
+  c.top2 = both(c.klim2 - 1u);
+  c.neg_top2 = both(1u - c.klim2);
+  c.neg_xe2 = both(0u - c.xe2);
+}
 __host__ __device__ __forceinline__ Clock make_clock(uint32_t tm, uint32_t k) {
   Clock c;
   const bool wrap = tm + 1u < k;
@@ -141,6 +153,7 @@ __host__ __device__ __forceinline__ Clock make_clock(uint32_t tm, uint32_t k) {
   c.klim2 = klim | (klim << 16);
   c.xe2 = xe | (xe << 16);
   c.wrap = wrap ? 1u : 0u;
+  fused_operands(c);
   return c;
 }
 __host__ __device__ __forceinline__ Clock distance_clock(uint32_t k) {
@@ -151,6 +164,7 @@ __host__ __device__ __forceinline__ Clock distance_clock(uint32_t k) {
   c.klim2 = k | (k << 16);
   c.xe2 = 0xFFFFFFFFu;   // never matched by a stored value that is advanced (no advance on distances)
   c.wrap = 0u;
+  fused_operands(c);
   return c;
 }
 // 0xFFFF in each half of a word whose recorder lies inside the window.
@@ -178,33 +192,27 @@ __device__ __forceinline__ uint4 set8(uint4 v, uint32_t t, uint32_t tm2) {
   return make_uint4(set2(v.x, t & 3u, tm2), set2(v.y, (t >> 2) & 3u, tm2), set2(v.z, (t >> 4) & 3u, tm2),
                     set2(v.w, t >> 6, tm2));
 }
-// The same tests with fewer instructions: a stamp lies inside a range [lo, hi] (lo <= hi) exactly
-// when clamping it into the range leaves it unchanged. The window is [lo, tm], or [lo, 65534] and
-// [0, tm] when it wraps (kNever lies in neither). min/max.u16x2 are single instructions on sm_90
-// and later, where the compares and subtractions of 16-bit halves above are not.
+// The same tests with fewer instructions, for the streaming passes: the packed 16-bit add with a
+// following minimum or maximum is one instruction on sm_90 and later (all of them, like min and max
+// alone, at 64 lanes per clock and SM here, where the pass has about 40 of them per 16-byte vector
+// before they, and not DRAM, bound it).
 __device__ __forceinline__ uint32_t umin2(uint32_t a, uint32_t b) {
   uint32_t r;
   asm("min.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
   return r;
 }
-__device__ __forceinline__ uint32_t umax2(uint32_t a, uint32_t b) {
-  uint32_t r;
-  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-  return r;
-}
-// 1 in each half of x outside [lo, hi], 0 inside.
-__device__ __forceinline__ uint32_t out_range2(uint32_t x, uint32_t lo2, uint32_t hi2) {
-  return umin2(umax2(umin2(x, hi2), lo2) ^ x, 0x00010001u);
-}
-// 1 in each half of x outside the window, 0 inside (so a sum of these words counts the recorders
-// outside, per half, in 16-bit fields). WRAP = c.wrap, chosen once per group by the caller (it is
-// the same for the whole grid), so the common case pays for one range only.
-template <bool WRAP>
+__device__ __forceinline__ uint32_t add_max2(uint32_t a, uint32_t b, uint32_t c) { return __viaddmax_u16x2(a, b, c); }
+__device__ __forceinline__ uint32_t add_min2(uint32_t a, uint32_t b, uint32_t c) { return __viaddmin_u16x2(a, b, c); }
+// 1 in each half of x outside the 16-bit range [lo, lo + klim) of the window, 0 inside (so a sum of
+// these words counts the recorders outside, per half, in 16-bit fields). When the window wraps,
+// kNever lies inside that range: not_never2 finds it.
 __device__ __forceinline__ uint32_t out2(uint32_t x, const Clock& c) {
-  uint32_t o = out_range2(x, c.lo2, c.hi2);
-  if (WRAP) o &= out_range2(x, 0u, c.tm2);
-  return o;
+  return add_min2(add_max2(x, c.neg_lo2, c.top2), c.neg_top2, 0x00010001u);
 }
+// 0 in each half of x that is kNever, 1 elsewhere.
+__device__ __forceinline__ uint32_t not_never2(uint32_t x) { return add_min2(x, 0x00010001u, 0x00010001u); }
+// Whether a half of x is 0.
+__device__ __forceinline__ bool zero_half(uint32_t x) { return umin2(x, 0x00010001u) != 0x00010001u; }
 // Whether any of the 8 recorders holds the stamp xe (a zero half in x ^ xe).
 __device__ __forceinline__ bool any_eq8(uint4 v, uint32_t xe2) {
   const uint32_t m = umin2(umin2(v.x ^ xe2, v.y ^ xe2), umin2(v.z ^ xe2, v.w ^ xe2));

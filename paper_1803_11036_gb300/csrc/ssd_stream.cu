@@ -39,6 +39,28 @@ __device__ __forceinline__ uint32_t lt8(uint4 v, uint32_t kk) {
 struct RouterClock {
   uint32_t tm2, xe2;
 };
+
+// Recorders at vector `at` of the n routers merged exactly, router by router: their distances at their
+// own clocks, the elementwise minimum; with ADV the vectors that hold an expiring recorder are
+// written back. The streaming pass calls it for the lanes its fused form cannot decide. Out of line: they
+// are rare.
+template <bool ADV>
+__device__ __noinline__ uint4 merge_exact(uint16_t* const* routers, const RouterClock* sck, int n, uint64_t at) {
+  uint4 mv = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    uint4* const p = reinterpret_cast<uint4*>(routers[j]) + at;
+    const uint4 v = __ldcg(p);
+    const RouterClock rc = sck[j];
+    mv = min8(mv, flip8(v, rc.tm2));
+    if (ADV) {
+      const uint4 e = make_uint4(__vcmpeq2(v.x, rc.xe2), __vcmpeq2(v.y, rc.xe2), __vcmpeq2(v.z, rc.xe2),
+                                 __vcmpeq2(v.w, rc.xe2));
+      if (any8(e)) __stcs(p, or8(v, e));
+    }
+  }
+  return mv;
+}
 __device__ __forceinline__ RouterClock router_clock(const uint32_t* tm) {
   RouterClock rc;
   const uint32_t t = read_tm(tm), xe = tm_next(t);
@@ -116,15 +138,18 @@ __device__ __forceinline__ void stcs_if(uint4* p, uint4 v, bool c) {
 // inside the window counted (out2), and the vectors that changed written back: a recorder set by
 // a touch, or, with ADV, one whose distance reaches 65535 at this advance (it becomes kNever).
 // The common path has no divergent branch: touched vectors are stored by predicated stores, and
-// the expiry (any_eq8 per vector) is taken once for the group behind a warp vote, reading back the
-// vectors it rewrites. No window bits are written: the caller builds them with group_bits only
-// for a hot estimator. Returns the lane's count of recorders inside the window.
+// the expiry is one running minimum of x - xe over the group, 0 when a recorder holds xe; the lanes
+// that see one read their vectors back and rewrite those. No window bits are written: the caller builds them with
+// group_bits only for a hot estimator. Returns the lane's count of recorders inside the window.
+// Four instructions per word: two fused ones and half an add for the window, one for
+// the expiry.
 template <bool ADV, bool HOT, bool TOUCH, bool WRAP>
 __device__ __forceinline__ uint32_t fast_group_w(uint4* r0, uint4* g, uint64_t base, uint32_t it0, uint32_t m,
                                                  int lane, const Clock& c, const uint4* tmask, uint4 (&v)[8],
                                                  uint64_t tw) {
-  uint32_t out = 0;   // recorders outside the window, per half, in two 16-bit fields
-  uint32_t expiring = 0;   // bit u: vector u holds a recorder with the stamp xe
+  uint32_t out = 0;   // recorders outside the window's range, per half, in two 16-bit fields
+  uint32_t set = 0;   // WRAP: recorders that are not kNever
+  uint32_t least = 0xFFFFFFFFu;   // least x - xe, per half
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     if (u < (int)m) {
@@ -135,19 +160,28 @@ __device__ __forceinline__ uint32_t fast_group_w(uint4* r0, uint4* g, uint64_t b
         stcs_if(r0 + at, v[u], t != 0u);
       }
       if (g) __stcs(g + at, v[u]);
-      if (HOT) out += out2<WRAP>(v[u].x, c) + out2<WRAP>(v[u].y, c) + out2<WRAP>(v[u].z, c) + out2<WRAP>(v[u].w, c);
-      if (ADV) expiring |= any_eq8(v[u], c.xe2) ? 1u << u : 0u;
-    }
-  }
-  if (ADV && __any_sync(kFull, expiring != 0u)) {   // once in 65535 slots per recorder
-    for (uint32_t u = 0; u < m; ++u) {
-      if ((expiring >> u) & 1u) {
-        const uint64_t at = base + (it0 + u) * 32 + lane;
-        __stcs(r0 + at, expire_vec(__ldcg(r0 + at), c.xe2));   // the lane's own (touched) vector
+      if (HOT) {
+        out += out2(v[u].x, c) + out2(v[u].y, c) + out2(v[u].z, c) + out2(v[u].w, c);
+        if (WRAP) set += not_never2(v[u].x) + not_never2(v[u].y) + not_never2(v[u].z) + not_never2(v[u].w);
+      }
+      if (ADV) {
+        least = add_min2(v[u].x, c.neg_xe2, least);
+        least = add_min2(v[u].y, c.neg_xe2, least);
+        least = add_min2(v[u].z, c.neg_xe2, least);
+        least = add_min2(v[u].w, c.neg_xe2, least);
       }
     }
   }
-  return 8u * m - (out & 0xFFFFu) - (out >> 16);
+  if (ADV && zero_half(least)) {   // once in 65535 slots per recorder
+#pragma unroll 1
+    for (uint32_t u = 0; u < m; ++u) {
+      const uint64_t at = base + (it0 + u) * 32 + lane;
+      const uint4 w = __ldcg(r0 + at);   // the lane's own (touched) vector
+      if (any_eq8(w, c.xe2)) __stcs(r0 + at, expire_vec(w, c.xe2));
+    }
+  }
+  const uint32_t in = WRAP ? set - out : both(4u * m) - out;   // per half (no borrow: out counts at most those)
+  return (in & 0xFFFFu) + (in >> 16);
 }
 // fast_group with the window's form chosen once for the group (c.wrap is the same for the grid).
 template <bool ADV, bool HOT, bool TOUCH>
@@ -160,8 +194,8 @@ __device__ __forceinline__ uint32_t fast_group(uint4* r0, uint4* g, uint64_t bas
 
 // The window bits of a group fast_group has processed, to `my`, from the recorders read again one
 // vector at a time (the lane reads back the vectors it stored itself; a hot estimator is rare, so
-// nothing is kept live in registers for it). A recorder the advance expired holds kNever, outside the window, as its
-// stamp xe was.
+// nothing is kept live in registers for it: eight loads in flight made the whole pass spill and cost more
+// than they gave). A recorder the advance expired holds kNever, outside the window, as its stamp xe was.
 __device__ __forceinline__ void group_bits(const uint4* r0, uint64_t base, uint32_t it0, uint32_t m, uint8_t* my,
                                            int lane, const Clock& c) {
 #pragma unroll 1
@@ -222,10 +256,17 @@ __device__ __forceinline__ void pool_if_hot(const Dims& d, const Scratch& s, uin
 }
 
 // eta >= 256: one warp per estimator, iters = eta/256 steps of 32 lanes x 8 recorders.
-// G (several routers): routers loaded per group before any of them is stored. One router works on
-// its stamps directly (window test, expiry); several routers are merged as distances (each
-// router's stamps through its own clock), and the global RSEA takes router 0's clock.
-template <bool ONE, bool ADV, bool HOT, bool TOUCH, int G>
+// One router works on its stamps directly (window test, expiry). Several routers are taken R at a time
+// over I steps, R * I vectors per lane loaded before any is used (fewer routers than 8 would
+// leave too few bytes in flight otherwise). When their clocks agree, which sketches
+// that advance together have, a stamp x is compared as p = x - (tm + 1): the newer the stamp the larger p, except
+// that kNever takes the place `never` = 65534 - tm between the stamps up to tm and the stale ones
+// above tm. The merge is then the running maximum of p, and the running minimum finds what that cannot decide: 0, a
+// recorder that expires; and a maximum of `never` with a smaller minimum, where a stale stamp is the
+// newest (only where it matters: a merged sketch is written, or the window wraps).
+// merge_exact takes those lanes, and every lane when the clocks differ. Two instructions per word and
+// router instead of about twelve: 32 routers of 1.25 GiB each went from 4.2 to over 6 TB/s, bound by DRAM.
+template <bool ONE, bool ADV, bool HOT, bool TOUCH, int R, int I>
 __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims d, const Scratch s,
                                                          const __grid_constant__ StreamArgs a) {
   extern __shared__ __align__(16) uint8_t smask[];
@@ -236,7 +277,6 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
   const uint64_t count = a.se_count ? a.se_count : ((uint64_t)d.r << d.q);
   const uint64_t se_end = a.se0 + count;
   const uint32_t iters = d.eta >> 8;
-  const uint32_t kk = d.k | (d.k << 16);
   const uint64_t wstride = (uint64_t)gridDim.x * (kBlock / 32);
   const uint64_t tstride = count * (d.eta >> 3);  // touch bytes per router
   uint4* const g = reinterpret_cast<uint4*>(a.global);
@@ -244,14 +284,22 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
   const uint32_t tm0 = read_tm(a.tm[0]);
   const Clock c = stamps ? make_clock(tm0, d.k) : distance_clock(d.k);
   if (a.global_tm && blockIdx.x == 0 && threadIdx.x == 0) *a.global_tm = tm0;
+  bool same = true;   // several routers: the clocks agree
   if (!ONE) {
-    for (int j = threadIdx.x; j < a.n; j += blockDim.x) sck[j] = router_clock(a.tm[j]);
-    __syncthreads();
+    for (int j = threadIdx.x; j < a.n; j += blockDim.x) {
+      sck[j] = router_clock(a.tm[j]);
+      same = same && sck[j].tm2 == c.tm2;
+    }
+    same = __syncthreads_and(same);
   }
   if (ONE && TOUCH) {
     for (int j = threadIdx.x; j < 256; j += blockDim.x) stm[j] = touch_mask_entry((uint32_t)j);
     __syncthreads();
   }
+  const uint32_t to_p = both(0u - (tm0 + 1u)), from_p = both(tm0 + 1u);
+  const uint32_t never2 = both(65534u - tm0);
+  Clock pc = c;   // the window test on p
+  pc.neg_lo2 = both(tm0 + 1u - c.lo2);
 
   for (uint64_t se = a.se0 + (uint64_t)blockIdx.x * (kBlock / 32) + wid; se < se_end; se += wstride) {
     const uint64_t base = (se << d.log2_eta) >> 3;  // in 8-recorder units
@@ -261,49 +309,90 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
       uint4* const r0 = reinterpret_cast<uint4*>(a.routers[0]);
       cnt = one_router_se<ADV, HOT, TOUCH>(d, r0, g, base, tb, my, lane, c, stm);
     } else {
-      for (uint32_t it = 0; it < iters; ++it) {
-        const uint64_t at = base + it * 32 + lane;
-        uint4 mv = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);   // distances
-        // routers in groups of G: the group's loads are issued before any of its stores
-        for (int n0 = 0; n0 < a.n; n0 += G) {
-          const int m = a.n - n0 < G ? a.n - n0 : G;
-          uint4 v[G];
-          uint32_t t[G];
+      for (uint32_t it0 = 0; it0 < iters; it0 += I) {
+        uint4 hi[I], lo[I];   // running maximum and minimum of p over the routers
 #pragma unroll
-          for (int u = 0; u < G; ++u) {
+        for (int i = 0; i < I; ++i) {
+          hi[i] = make_uint4(0u, 0u, 0u, 0u);
+          lo[i] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+        }
+        // routers in groups of R: the group's loads are issued before any of its stores
+        for (int n0 = 0; n0 < a.n; n0 += R) {
+          const int m = a.n - n0 < R ? a.n - n0 : R;
+          uint4 v[R][I];
+#pragma unroll
+          for (int u = 0; u < R; ++u) {
             if (u < m) {
-              v[u] = __ldcs(reinterpret_cast<uint4*>(a.routers[n0 + u]) + at);
-              if (TOUCH) t[u] = tb[(uint64_t)(n0 + u) * tstride + it];
+              const uint4* const p = reinterpret_cast<const uint4*>(a.routers[n0 + u]) + base + lane;
+#pragma unroll
+              for (int i = 0; i < I; ++i)
+                if (I == 1 || it0 + i < iters) v[u][i] = __ldcs(p + (it0 + i) * 32);
             }
           }
 #pragma unroll
-          for (int u = 0; u < G; ++u) {
+          for (int u = 0; u < R; ++u) {
             if (u < m) {
-              const RouterClock rc = sck[n0 + u];
-              bool dirty = false;
-              if (TOUCH && t[u]) {
-                v[u] = set8(v[u], t[u], rc.tm2);
-                tb[(uint64_t)(n0 + u) * tstride + it] = 0;
-                dirty = true;
-              }
-              mv = min8(mv, stamps ? flip8(v[u], rc.tm2) : v[u]);
-              if (ADV) {
-                const uint4 e = make_uint4(__vcmpeq2(v[u].x, rc.xe2), __vcmpeq2(v[u].y, rc.xe2),
-                                           __vcmpeq2(v[u].z, rc.xe2), __vcmpeq2(v[u].w, rc.xe2));
-                if (any8(e)) {
-                  v[u] = or8(v[u], e);
-                  dirty = true;
+#pragma unroll
+              for (int i = 0; i < I; ++i) {
+                if (I > 1 && it0 + i >= iters) continue;
+                if (TOUCH) {
+                  uint8_t* const t8 = tb + (uint64_t)(n0 + u) * tstride + it0 + i;
+                  const uint32_t t = *t8;
+                  if (t) {
+                    *t8 = 0;
+                    v[u][i] = set8(v[u][i], t, sck[n0 + u].tm2);
+                    __stcs(reinterpret_cast<uint4*>(a.routers[n0 + u]) + base + (it0 + i) * 32 + lane, v[u][i]);
+                  }
                 }
+                const uint4 x = v[u][i];
+                if (HOT || g) {
+                  hi[i] = make_uint4(add_max2(x.x, to_p, hi[i].x), add_max2(x.y, to_p, hi[i].y),
+                                     add_max2(x.z, to_p, hi[i].z), add_max2(x.w, to_p, hi[i].w));
+                }
+                lo[i] = make_uint4(add_min2(x.x, to_p, lo[i].x), add_min2(x.y, to_p, lo[i].y),
+                                   add_min2(x.z, to_p, lo[i].z), add_min2(x.w, to_p, lo[i].w));
               }
-              if (dirty) __stcs(reinterpret_cast<uint4*>(a.routers[n0 + u]) + at, v[u]);
             }
           }
         }
-        if (g) __stcs(g + at, stamps ? flip8(mv, c.tm2) : mv);
-        if (HOT) {
-          const uint32_t bits = lt8(mv, kk);
-          cnt += __popc(bits);
-          my[it * 32 + lane] = (uint8_t)bits;
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+          if (I > 1 && it0 + i >= iters) continue;
+          const uint64_t at = base + (it0 + i) * 32 + lane;
+          bool exact = !same;
+          // at tm = 65534 kNever is p = 0 and the expiring stamp 0 is p = 1: every lane with a 0 is taken
+          if (ADV) exact = exact || zero_half(umin2(umin2(lo[i].x, lo[i].y), umin2(lo[i].z, lo[i].w)));
+          if (ADV && tm0 == 65534u) exact = true;
+          if ((HOT && c.wrap) || g) {
+            // 1 in a half whose maximum is `never` while its minimum differs
+            auto stale = [&](uint32_t h, uint32_t l) {
+              return umin2(h ^ l, 0x00010001u) & ~umin2(h ^ never2, 0x00010001u);
+            };
+            exact = exact || ((stale(hi[i].x, lo[i].x) | stale(hi[i].y, lo[i].y) | stale(hi[i].z, lo[i].z) |
+                               stale(hi[i].w, lo[i].w)) & 0x00010001u) != 0u;
+          }
+          if (exact) {
+            const uint4 mv = flip8(merge_exact<ADV>(a.routers, sck, a.n, at), c.tm2);   // stamps at clock tm0
+            hi[i] = make_uint4(__vadd2(mv.x, to_p), __vadd2(mv.y, to_p), __vadd2(mv.z, to_p), __vadd2(mv.w, to_p));
+          }
+          if (g)
+            __stcs(g + at, make_uint4(__vadd2(hi[i].x, from_p), __vadd2(hi[i].y, from_p), __vadd2(hi[i].z, from_p),
+                                      __vadd2(hi[i].w, from_p)));
+          if (HOT) {
+            // one bit per recorder (0: inside the window), words interleaved: bitmaps are only ever
+            // compared with others of the same pass, so the order of their bits is free
+            uint32_t o[4] = {out2(hi[i].x, pc), out2(hi[i].y, pc), out2(hi[i].z, pc), out2(hi[i].w, pc)};
+            if (c.wrap) {   // kNever lies in the range of a window that wraps
+              o[0] |= umin2(hi[i].x ^ never2, 0x00010001u) ^ 0x00010001u;
+              o[1] |= umin2(hi[i].y ^ never2, 0x00010001u) ^ 0x00010001u;
+              o[2] |= umin2(hi[i].z ^ never2, 0x00010001u) ^ 0x00010001u;
+              o[3] |= umin2(hi[i].w ^ never2, 0x00010001u) ^ 0x00010001u;
+            }
+            const uint32_t in = (o[0] + 2u * o[1] + 4u * o[2] + 8u * o[3]) ^ 0x000F000Fu;
+            const uint32_t bits = (in | (in >> 12)) & 0xFFu;
+            cnt += __popc(bits);
+            my[(it0 + i) * 32 + lane] = (uint8_t)bits;
+          }
         }
       }
     }
@@ -532,14 +621,14 @@ int blocks_per_sm(K kernel, size_t smem, const Tuning& tn) {
   return b > 0 ? b : 1;
 }
 
-template <bool ONE, bool ADV, bool HOT, bool TOUCH, int G>
+template <bool ONE, bool ADV, bool HOT, bool TOUCH, int R, int I>
 cudaError_t launch_large(const Dims& d, const Scratch& s, const StreamArgs& a, uint64_t count, int sms,
                          const Tuning& tn, cudaStream_t st) {
   const size_t smem = HOT ? (size_t)(kBlock / 32) * (d.eta >> 3) : 0;
   const uint64_t need = (count + (kBlock / 32) - 1) / (kBlock / 32);
-  uint64_t grid = (uint64_t)sms * blocks_per_sm(k_stream_large<ONE, ADV, HOT, TOUCH, G>, smem, tn);
+  uint64_t grid = (uint64_t)sms * blocks_per_sm(k_stream_large<ONE, ADV, HOT, TOUCH, R, I>, smem, tn);
   if (grid > need) grid = need;
-  k_stream_large<ONE, ADV, HOT, TOUCH, G><<<(unsigned)grid, kBlock, smem, st>>>(d, s, a);
+  k_stream_large<ONE, ADV, HOT, TOUCH, R, I><<<(unsigned)grid, kBlock, smem, st>>>(d, s, a);
   return cudaGetLastError();
 }
 
@@ -548,10 +637,21 @@ cudaError_t launch_variant(const Dims& d, const Scratch& s, const StreamArgs& a,
                            cudaStream_t st) {
   const uint64_t count = a.se_count ? a.se_count : ((uint64_t)d.r << d.q);
   if (d.eta >= 256) {
-    if (ONE) return launch_large<ONE, ADV, HOT, TOUCH, 1>(d, s, a, count, sms, tn, st);
-    if (tn.group == 2) return launch_large<ONE, ADV, HOT, TOUCH, 2>(d, s, a, count, sms, tn, st);
-    if (tn.group == 4) return launch_large<ONE, ADV, HOT, TOUCH, 4>(d, s, a, count, sms, tn, st);
-    return launch_large<ONE, ADV, HOT, TOUCH, 8>(d, s, a, count, sms, tn, st);
+    if constexpr (ONE) {
+      return launch_large<true, ADV, HOT, TOUCH, 1, 1>(d, s, a, count, sms, tn, st);
+    } else {
+      // tn.group vectors per lane in flight. Several consecutive ones of fewer routers where an
+      // estimator has them: 4 x 2 reads 1 KB of a router at a time, and 16 and 32 routers then stream at
+      // 7.3 TB/s where 8 x 1 (512 B) reaches 6.0
+      if (tn.group == 2) return launch_large<false, ADV, HOT, TOUCH, 2, 1>(d, s, a, count, sms, tn, st);
+      if (tn.group == 4) {
+        if (d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 2, 2>(d, s, a, count, sms, tn, st);
+        return launch_large<false, ADV, HOT, TOUCH, 4, 1>(d, s, a, count, sms, tn, st);
+      }
+      if (a.n == 2 && d.eta >= 1024) return launch_large<false, ADV, HOT, TOUCH, 2, 4>(d, s, a, count, sms, tn, st);
+      if (d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 4, 2>(d, s, a, count, sms, tn, st);
+      return launch_large<false, ADV, HOT, TOUCH, 8, 1>(d, s, a, count, sms, tn, st);
+    }
   }
   const uint64_t n_units = count * d.eta / 256;
   const uint64_t need = (n_units + (kBlock / 32) - 1) / (kBlock / 32);
