@@ -193,12 +193,17 @@ int stream_pass(ssd_ctx* ctx, ssd_sketch* const* routers, int n, ssd_sketch* glo
   return SSD_OK;
 }
 
-// The clocks of advanced sketches move on by one slot, after every launch that reads them.
-int tick(ssd_ctx* ctx, ssd_sketch* const* sketches, int n, cudaStream_t st) {
+ssd::TickArgs tick_args(ssd_sketch* const* sketches, int n) {
   ssd::TickArgs a;
   std::memset(&a, 0, sizeof(a));
   a.n = n;
   for (int i = 0; i < n; ++i) a.tm[i] = sketches[i]->tm;
+  return a;
+}
+
+// The clocks of advanced sketches move on by one slot, after every launch that reads them.
+int tick(ssd_ctx* ctx, ssd_sketch* const* sketches, int n, cudaStream_t st) {
+  const ssd::TickArgs a = tick_args(sketches, n);
   cudaError_t e = ssd::launch_tick(a, st);
   if (e != cudaSuccess) return cuda_fail(e, "tick kernel");
   ctx->launches += 1;
@@ -244,11 +249,13 @@ int trace(ssd_ctx* ctx, cudaEvent_t ev, cudaStream_t st) {
   return e == cudaSuccess ? SSD_OK : cuda_fail(e, "cudaEventRecord (trace)");
 }
 
+// The regain after a kHot pass; the clocks of the n `ticking` sketches move on with its last launch.
 int regain_after_pass(ssd_ctx* ctx, uint32_t* ips, uint32_t* rk, uint64_t cap, unsigned long long* n_out,
-                      cudaStream_t st, uint32_t view) {
+                      cudaStream_t st, uint32_t view, ssd_sketch* const* ticking = nullptr, int n = 0) {
   int launches = 0;
+  const ssd::TickArgs ticks = tick_args(ticking, n);
   cudaError_t e = ssd::launch_regain_tail(ctx->d, ctx->s, ips, rk, cap, n_out, ctx->sms, st, &launches, view,
-                                          ctx->tn.pair_level == 0);
+                                          ctx->tn.pair_level == 0, &ticks);
   ctx->launches += launches;
   if (e != cudaSuccess) return cuda_fail(e, "regain kernels");
   return SSD_OK;
@@ -760,8 +767,7 @@ int ssd_close_slot(ssd_ctx* ctx, ssd_sketch* const* routers, int n, ssd_sketch* 
   rc = stream_pass(ctx, routers, n, global, ssd::kAdvance | ssd::kHot, st);
   if (rc == SSD_OK) rc = trace(ctx, ctx->tr_pass, st);
   unsigned long long* nd = d_n_out ? reinterpret_cast<unsigned long long*>(d_n_out) : ctx->n_out;
-  if (rc == SSD_OK) rc = regain_after_pass(ctx, d_ips, d_rk, cap, nd, st, routers[0]->view);
-  if (rc == SSD_OK) rc = tick(ctx, routers, n, st);
+  if (rc == SSD_OK) rc = regain_after_pass(ctx, d_ips, d_rk, cap, nd, st, routers[0]->view, routers, n);
   if (rc == SSD_OK) rc = trace(ctx, ctx->tr_end, st);
   if (rc != SSD_OK) return rc;
   const uint64_t merged = routers[0]->slot;
@@ -932,8 +938,7 @@ static int slot_chunks1(ssd_ctx* ctx, ssd_sketch* router, const uint32_t* pairs,
   }
   rc = trace(ctx, ctx->tr_pass, st);
   unsigned long long* nd = d_n_out ? reinterpret_cast<unsigned long long*>(d_n_out) : ctx->n_out;
-  if (rc == SSD_OK) rc = regain_after_pass(ctx, d_ips, d_rk, cap, nd, st, router->view);
-  if (rc == SSD_OK) rc = tick(ctx, &router, 1, st);
+  if (rc == SSD_OK) rc = regain_after_pass(ctx, d_ips, d_rk, cap, nd, st, router->view, &router, 1);
   if (rc == SSD_OK) rc = trace(ctx, ctx->tr_end, st);
   if (rc != SSD_OK) return rc;
   if (global) {
@@ -1019,8 +1024,7 @@ int ssd_slot(ssd_ctx* ctx, ssd_sketch* const* routers, const uint32_t* const* d_
   }
   rc = trace(ctx, ctx->tr_pass, st);
   unsigned long long* nd = d_n_out ? reinterpret_cast<unsigned long long*>(d_n_out) : ctx->n_out;
-  if (rc == SSD_OK) rc = regain_after_pass(ctx, d_ips, d_rk, cap, nd, st, routers[0]->view);
-  if (rc == SSD_OK) rc = tick(ctx, routers, n, st);
+  if (rc == SSD_OK) rc = regain_after_pass(ctx, d_ips, d_rk, cap, nd, st, routers[0]->view, routers, n);
   if (rc == SSD_OK) rc = trace(ctx, ctx->tr_end, st);
   if (rc != SSD_OK) return rc;
   const uint64_t merged = routers[0]->slot;

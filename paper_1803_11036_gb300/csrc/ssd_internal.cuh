@@ -483,8 +483,9 @@ cudaError_t launch_occupancy(const Dims& d, const uint16_t* dr, const uint32_t* 
 // Candidate levels, final test and the list; reads the pools filled by a kHot pass.
 // `view`: the regained sketch's view; hosts outside its group are not listed.
 // tensor_pairs: the pair level on the tensor cores when eta is a multiple of 128 and pruning is on.
+// tick: clocks that the last launch moves on by one slot.
 cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, uint32_t* rk, uint64_t cap,
                                unsigned long long* n_out_dev, int sms, cudaStream_t st, int* launches,
-                               uint32_t view = 0, bool tensor_pairs = false);
+                               uint32_t view = 0, bool tensor_pairs = false, const TickArgs* tick = nullptr);
 
 }  // namespace ssd

@@ -9,7 +9,7 @@
 //   the bitmaps expanded to bytes on the tensor cores (k_pairs_tc, the default
 //   for eta a multiple of 128), or as 64 x 64 tiles of AND-popcounts on the CUDA
 //   cores (4 x 4 per thread, one carry-save step per two words) with the bitmaps
-//   staged in shared memory; one append per tile either way.
+//   staged in shared memory; one append per tile either way. Few pairs skip the tiles.
 // Level i >= 2: the overlap test fixes the low q-delta bits of he_i
 //   (B(i) mod 2^(q-delta) = B(i-1) >> delta with B(j) = he_0 XOR he_j), so the
 //   only row-i estimators a candidate can extend to are the hot ones with those
@@ -93,43 +93,53 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Row i's pooled hot estimators bucketed by the low q-delta bits of their column
-// (one block; counting sort in global memory: count, exclusive scan, fill). The
-// order inside a bucket is that of the fill's atomics; the levels do not depend
-// on it (the list is sorted at the end).
-__device__ void build_buckets(const Dims& d, const Scratch& s, uint32_t i) {
-  __shared__ uint32_t part[kBlock];
+// Row i's pooled hot estimators bucketed by the low q-delta bits of their column (one block; counting
+// sort: count, exclusive scan, fill). The counters are kept in the `room` words of shared memory at `sm` where
+// they fit (six barriers and no round trip to L2 in between: about 5 us where 8192 counters in global
+// memory took 20), else in global memory. The order inside a bucket is that of the fill's atomics; the levels
+// do not depend on it (the list is sorted at the end).
+__device__ void build_buckets(const Dims& d, const Scratch& s, uint32_t i, uint32_t* sm, uint32_t room) {
+  __shared__ uint32_t part[kBlock / 32];
   const uint32_t nb = 1u << d.low_bits;
   uint32_t* off = s.bucket_off + (uint64_t)i * (nb + 1);
-  uint32_t* cnt = s.bucket_cnt + (uint64_t)i * nb;
+  uint32_t* cnt = nb <= room ? sm : s.bucket_cnt + (uint64_t)i * nb;
   uint32_t* ent = s.bucket_ent + (uint64_t)i * d.hse_cap;
   const uint32_t* col = s.pool_col + (uint64_t)i * d.hse_cap;
   const uint32_t n = min(s.counters->hot[i], d.hse_cap);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) cnt[b] = 0;
   __syncthreads();
   for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) atomicAdd(&cnt[col[j] & d.low_mask], 1u);
   __syncthreads();
-  // exclusive scan: each thread sums a contiguous segment, the block scans the sums
-  const uint32_t seg = (nb + blockDim.x - 1) / blockDim.x;
-  const uint32_t lo = min(threadIdx.x * seg, nb), hi = min(lo + seg, nb);
-  uint32_t sum = 0;
-  for (uint32_t b = lo; b < hi; ++b) sum += cnt[b];
-  part[threadIdx.x] = sum;
-  __syncthreads();
-  for (uint32_t o = 1; o < blockDim.x; o <<= 1) {   // inclusive Hillis-Steele scan of the sums
-    const uint32_t v = threadIdx.x >= o ? part[threadIdx.x - o] : 0u;
+  // exclusive scan by steps of a block: each warp takes 32 consecutive counters of a step, so that reads
+  // and writes coalesce
+  uint32_t run = 0;
+  for (uint32_t b0 = 0; b0 < nb; b0 += kBlock) {
+    const uint32_t b = b0 + threadIdx.x;
+    const uint32_t c = b < nb ? cnt[b] : 0u;
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) part[wid] = incl;
     __syncthreads();
-    part[threadIdx.x] += v;
-    __syncthreads();
+    uint32_t before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kBlock / 32; ++w) {
+      before += w < wid ? part[w] : 0u;
+      total += part[w];
+    }
+    if (b < nb) {
+      const uint32_t at = run + before + incl - c;
+      off[b] = at;
+      cnt[b] = at;   // the fill's cursor
+    }
+    run += total;
+    __syncthreads();   // part is reused by the next step
   }
-  uint32_t run = threadIdx.x ? part[threadIdx.x - 1] : 0u;
-  for (uint32_t b = lo; b < hi; ++b) {
-    const uint32_t c = cnt[b];
-    off[b] = run;
-    cnt[b] = run;   // the fill's cursor
-    run += c;
-  }
-  if (threadIdx.x == blockDim.x - 1) off[nb] = part[blockDim.x - 1];
+  if (threadIdx.x == 0) off[nb] = run;
   __syncthreads();
   for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) ent[atomicAdd(&cnt[col[j] & d.low_mask], 1u)] = j;
 }
@@ -151,11 +161,11 @@ __device__ __forceinline__ uint32_t csa_pop(uint32_t& ones, uint32_t a, uint32_t
 // row 2 + m.
 __global__ void __launch_bounds__(kBlock, 3) k_pairs(const Dims d, const Scratch s, uint32_t pair_blocks) {
   pdl_enter();
+  __shared__ uint32_t A[TA][KW + 1], B[TA][KW + 1];
   if (blockIdx.x >= pair_blocks) {
-    build_buckets(d, s, 2 + (blockIdx.x - pair_blocks));
+    build_buckets(d, s, 2 + (blockIdx.x - pair_blocks), &A[0][0], TA * (KW + 1));
     return;
   }
-  __shared__ uint32_t A[TA][KW + 1], B[TA][KW + 1];
   __shared__ uint32_t wsum[kBlock / 32];
   __shared__ unsigned long long tile_base;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -367,22 +377,92 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
       : "memory");
 }
 
+// At most this many pairs are tested one by one: spread over every warp of the grid, a pair costs eight lanes
+// a few loads, and 40 K pairs of 2048-recorder estimators (20 MB of L2 reads) take 6 us, where the few
+// tiles they make keep a few blocks busy for 16 dependent stages and more (20 x 20 pairs: 15 us, 200 x 200:
+// 17 us). Past about 130 K pairs the tiles, which read each bitmap once per tile, are faster.
+constexpr uint64_t kDirectPairs = 1u << 18;
+__device__ __forceinline__ void pairs_direct(const Dims& d, const Scratch& s, uint32_t n0, uint32_t n1,
+                                             uint32_t blocks) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t grp = lane >> 3, gl = lane & 7u;
+  const uint32_t warps = blocks * (kTcThreads / 32), gw = blockIdx.x * (kTcThreads / 32) + (threadIdx.x >> 5);
+  const uint32_t total = n0 * n1, vecs = d.words >> 2;
+  const uint4* const bm0 = reinterpret_cast<const uint4*>(s.pool_bm);
+  const uint4* const bm1 = bm0 + (uint64_t)d.hse_cap * vecs;
+  constexpr int U = 4;   // pairs per group of lanes in flight
+  for (uint32_t p0 = gw * 4 * U; p0 < total; p0 += warps * 4 * U) {
+    uint32_t pa[U], pb[U], rk[U];
+    bool keep[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t p = p0 + u * 4 + grp;
+      const bool live = p < total;
+      pa[u] = live ? p / n1 : 0u;
+      pb[u] = live ? p - pa[u] * n1 : 0u;
+      rk[u] = 0;
+    }
+    for (uint32_t v = gl; v < vecs; v += 8) {
+      uint4 x[U], y[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        x[u] = bm0[(uint64_t)pa[u] * vecs + v];
+        y[u] = bm1[(uint64_t)pb[u] * vecs + v];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        rk[u] += __popc(x[u].x & y[u].x) + __popc(x[u].y & y[u].y) + __popc(x[u].z & y[u].z) + __popc(x[u].w & y[u].w);
+    }
+    unsigned n = 0, mine = 0;
+    unsigned masks[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) rk[u] += __shfl_xor_sync(kFull, rk[u], o);
+      keep[u] = gl == 0 && p0 + u * 4 + grp < total && rk[u] >= d.thr;
+      masks[u] = __ballot_sync(kFull, keep[u]);
+      n += __popc(masks[u]);
+    }
+    if (!n) continue;   // warp-uniform
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(&s.counters->level[1], (unsigned long long)n);
+    base = __shfl_sync(kFull, base, 0);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (keep[u]) {
+        const unsigned long long pos = base + mine + __popc(masks[u] & ((1u << lane) - 1u));
+        if (pos < d.ctb_cap) {
+          s.ctb[0][pos * d.r + 0] = pa[u];
+          s.ctb[0][pos * d.r + 1] = pb[u];
+        } else {
+          atomicOr(&s.counters->status, SSD_STATUS_CTB_OVERFLOW);
+        }
+      }
+      mine += __popc(masks[u]);
+    }
+  }
+}
+
 // Blocks [0, tile_blocks) take the 128 x 256 tiles of HSE(0) x HSE(1) in turn (block b: tiles
 // b, b + tile_blocks, ...), with one tensor-memory allocation for all of them; with the bucket
 // index, block tile_blocks + m builds the buckets of row 2 + m (as in k_pairs). Needs eta a
 // multiple of 128 and pruning on (the caller checks).
 __global__ void __launch_bounds__(kTcThreads, 1) k_pairs_tc(const Dims d, const Scratch s, uint32_t tile_blocks) {
   pdl_enter();
+  extern __shared__ uint8_t tc_raw[];
   if (blockIdx.x >= tile_blocks) {
-    build_buckets(d, s, 2 + (blockIdx.x - tile_blocks));
+    build_buckets(d, s, 2 + (blockIdx.x - tile_blocks), reinterpret_cast<uint32_t*>(tc_raw), kTcSmem / 4);
     return;
   }
   const uint32_t n0 = min(s.counters->hot[0], d.hse_cap);
   const uint32_t n1 = min(s.counters->hot[1], d.hse_cap);
+  if ((uint64_t)n0 * n1 <= kDirectPairs) {
+    pairs_direct(d, s, n0, n1, tile_blocks);
+    return;
+  }
   const uint32_t tn = (n1 + kTcN - 1) / kTcN;
   const uint32_t ntiles = ((n0 + kTcM - 1) / kTcM) * tn;
   if (blockIdx.x >= ntiles) return;   // block-uniform: nothing allocated yet
-  extern __shared__ uint8_t tc_raw[];
   __shared__ __align__(8) uint64_t bar[3];   // stage buffer 0, stage buffer 1, a tile's MMAs done
   __shared__ uint32_t tmem_base;
   __shared__ uint32_t wsum[kTcThreads / 32];
@@ -635,6 +715,42 @@ __device__ __forceinline__ void stage_host(const Dims& d, const Scratch& s, bool
   }
 }
 
+// The last row's test of the warp's hits (idx extends tuple tl to row i = r - 1, the union has R_k pc): the
+// count, and for an accepted tuple the host and its staging. Every lane of the warp makes the call.
+__device__ __forceinline__ void last_hit(const Dims& d, const Scratch& s, uint32_t i, const uint32_t (&tl)[SSD_MAX_R],
+                                         uint32_t idx, uint32_t pc, uint32_t view) {
+  const uint64_t cap = d.hse_cap;
+  const bool prune = !(d.flags & SSD_NO_PRUNE);
+  const bool verify = (d.flags & SSD_VERIFY_H0) != 0;
+  const bool hit = idx != kNone;
+  warp_append(hit && (!prune || pc >= d.thr), &s.counters->level[i]);
+  bool acc = hit && pc >= d.thr;
+  uint32_t cip = 0, he0 = 0;
+  if (acc) {
+    uint32_t he[SSD_MAX_R];
+#pragma unroll
+    for (uint32_t j = 0; j < SSD_MAX_R; ++j) he[j] = j < i ? s.pool_col[(uint64_t)j * cap + tl[j]] : 0u;
+    const uint32_t last = s.pool_col[(uint64_t)i * cap + idx];
+#pragma unroll
+    for (uint32_t j = 0; j < SSD_MAX_R; ++j)
+      if (j == i) he[j] = last;
+    acc = regain_host(d, he, &cip);
+    he0 = he[0];
+  }
+  if (d.sh0 == 0) {
+    if (acc && verify) acc = (tab_hash_global(s.tables + 1024, cip) & d.col_mask) == he0;
+    if (acc) acc = view_host_in(view, cip);   // a grouped sketch holds only its group's hosts
+    stage_host(d, s, acc, cip, pc);
+  } else if (__any_sync(kFull, acc)) {
+    // Eq. 2 as printed: every completion of bits 0..delta-1 whose RHFG[0] is he_0
+    for (uint32_t low = 0; low < (1u << d.delta); ++low) {
+      const uint32_t x = cip | low;
+      const bool ok = acc && (tab_hash_global(s.tables + 1024, x) & d.col_mask) == he0 && view_host_in(view, x);
+      stage_host(d, s, ok, x, pc);
+    }
+  }
+}
+
 // One candidate tuple c (its pool indices tl, rows 0..i-1) of row level i
 // extended by row-i estimator idx (pool index; kNone when this lane has none):
 // the union test, then the append to the next candidate buffer or, at the last
@@ -642,10 +758,8 @@ __device__ __forceinline__ void stage_host(const Dims& d, const Scratch& s, bool
 // the call (the test and the appends are warp-wide).
 __device__ __forceinline__ void level_hit(const Dims& d, const Scratch& s, uint32_t i, uint32_t* sctb,
                                           const uint32_t (&tl)[SSD_MAX_R], uint32_t idx, int lane, uint32_t view) {
-  const uint64_t cap = d.hse_cap;
   const bool last = (i == d.r - 1);
   const bool prune = !(d.flags & SSD_NO_PRUNE);
-  const bool verify = (d.flags & SSD_VERIFY_H0) != 0;
   const bool hit = idx != kNone;
   const uint32_t pc = (prune || last) ? union_rk(d, s, i, tl, idx, lane) : 0u;
   const bool keep = hit && (!prune || pc >= d.thr);
@@ -662,30 +776,7 @@ __device__ __forceinline__ void level_hit(const Dims& d, const Scratch& s, uint3
       }
     }
   } else {
-    warp_append(keep, &s.counters->level[i]);
-    bool acc = hit && pc >= d.thr;
-    uint32_t cip = 0, he0 = 0;
-    if (acc) {
-      uint32_t he[SSD_MAX_R];
-#pragma unroll
-      for (uint32_t j = 0; j < SSD_MAX_R; ++j)
-        if (j < i) he[j] = s.pool_col[(uint64_t)j * cap + tl[j]];
-      he[i] = s.pool_col[(uint64_t)i * cap + idx];
-      acc = regain_host(d, he, &cip);
-      he0 = he[0];
-    }
-    if (d.sh0 == 0) {
-      if (acc && verify) acc = (tab_hash_global(s.tables + 1024, cip) & d.col_mask) == he0;
-      if (acc) acc = view_host_in(view, cip);   // a grouped sketch holds only its group's hosts
-      stage_host(d, s, acc, cip, pc);
-    } else if (__any_sync(kFull, acc)) {
-      // Eq. 2 as printed: every completion of bits 0..delta-1 whose RHFG[0] is he_0
-      for (uint32_t low = 0; low < (1u << d.delta); ++low) {
-        const uint32_t x = cip | low;
-        const bool ok = acc && (tab_hash_global(s.tables + 1024, x) & d.col_mask) == he0 && view_host_in(view, x);
-        stage_host(d, s, ok, x, pc);
-      }
-    }
+    last_hit(d, s, i, tl, idx, pc, view);
   }
 }
 
@@ -752,30 +843,128 @@ __global__ void __launch_bounds__(kBlock) k_level(const Dims d, const Scratch s,
   }
 }
 
-constexpr int kListThreads = 1024;
-constexpr uint32_t kSmemKeys = 16384;
+// The bucket of row-i hot estimators a tuple (rows 0..i-1) can extend to, as a range of bucket_ent.
+__device__ __forceinline__ uint2 extensions(const Dims& d, const Scratch& s, uint32_t i, uint32_t he0,
+                                            const uint32_t (&tl)[SSD_MAX_R]) {
+  uint32_t tp = 0;
+#pragma unroll
+  for (uint32_t j = 0; j < SSD_MAX_R; ++j)
+    if (j == i - 1) tp = tl[j];
+  const uint32_t hep = s.pool_col[(uint64_t)(i - 1) * d.hse_cap + tp];
+  const uint32_t low = (he0 ^ ((he0 ^ hep) >> d.delta)) & d.low_mask;
+  const uint32_t* off = s.bucket_off + (uint64_t)i * ((1u << d.low_bits) + 1);
+  const uint2 be = make_uint2(off[low], off[low + 1]);
+  return in_bounds(d, be.x <= be.y && be.y <= d.hse_cap) ? be : make_uint2(0u, 0u);
+}
 
-__device__ void bitonic(unsigned long long* keys, uint32_t P) {
-  for (uint32_t k = 2; k <= P; k <<= 1) {
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
-        const uint32_t ixj = i ^ j;
-        if (ixj > i) {
-          const unsigned long long a = keys[i], b = keys[ixj];
-          const bool up = (i & k) == 0;
-          if ((a > b) == up) { keys[i] = b; keys[ixj] = a; }
-        }
+// The tuples of the warp's `active` lanes (rows 0..I-1) extended through rows I .. r-1, depth first: a
+// kept extension goes on to the next row at once, in its lane, and is counted where the level-by-level
+// form would append it (a count past the candidate buffer's capacity is an overflow there, and
+// here).
+// A lane takes the entries first, first + step, ... of its bucket.
+template <uint32_t I>
+__device__ __forceinline__ void extend_rows(const Dims& d, const Scratch& s, uint32_t (&tl)[SSD_MAX_R], uint32_t he0,
+                                            bool active, int lane, uint32_t view, uint32_t first, uint32_t step) {
+  uint2 be = make_uint2(0u, 0u);
+  if (active) be = extensions(d, s, I, he0, tl);
+  be.x += first;
+  const uint32_t* ent = s.bucket_ent + (uint64_t)I * d.hse_cap;
+  for (; __any_sync(kFull, be.x < be.y); be.x += step) {
+    const uint32_t idx = be.x < be.y ? ent[be.x] : kNone;
+    const uint32_t pc = union_rk(d, s, I, tl, idx, lane);
+    if (I == d.r - 1) {
+      last_hit(d, s, I, tl, idx, pc, view);
+    } else if constexpr (I + 1 < SSD_MAX_R) {
+      bool keep = idx != kNone && pc >= d.thr;
+      const unsigned long long pos = warp_append(keep, &s.counters->level[I]);
+      if (keep && pos >= d.ctb_cap) {
+        atomicOr(&s.counters->status, SSD_STATUS_CTB_OVERFLOW);
+        keep = false;
       }
-      __syncthreads();
+      if (__any_sync(kFull, keep)) {
+        tl[I] = keep ? idx : 0u;
+        extend_rows<I + 1>(d, s, tl, he0, keep, lane, view, 0u, 1u);
+      }
     }
   }
 }
 
-// One block: sort the staged (cip << 32 | R_k) keys, keep the last entry of each
-// cip (its largest R_k), and write the list when it fits the caller's capacity.
-__global__ void __launch_bounds__(kListThreads) k_list(const Dims d, const Scratch s, uint32_t* ips, uint32_t* rk,
-                                                       uint64_t cap, unsigned long long* n_out_dev) {
+// Rows 2 .. r-1 in one launch (pruning on, bucket index there): the pairs that survived are few
+// and their extensions fewer, so a launch per row was three times the latency of one (candidate,
+// bucket, bitmaps, append) and little work. Bound by that latency chain.
+__global__ void __launch_bounds__(kBlock) k_extend(const Dims d, const Scratch s, const uint32_t view) {
   pdl_enter();
+  const int lane = threadIdx.x & 31;
+  const unsigned long long avail = s.counters->level[1];
+  const uint64_t nc = avail < d.ctb_cap ? avail : d.ctb_cap;
+  // few candidates: several lanes share one (each takes a part of its row-2 bucket), so that all warps have work
+  const uint64_t threads = (uint64_t)gridDim.x * blockDim.x;
+  uint32_t share = 1;
+  while (share < 32 && nc * share * 2 <= threads) share *= 2;
+  const uint64_t stride = threads / share;
+  const uint32_t per_warp = 32 / share;
+  uint32_t tl[SSD_MAX_R];
+#pragma unroll
+  for (uint32_t j = 0; j < SSD_MAX_R; ++j) tl[j] = 0;
+  // warps in the order of their SMs' first blocks: warp w of block b is the (w * blocks + b)-th
+  const uint64_t warp = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  for (uint64_t w0 = warp * per_warp; w0 < nc; w0 += stride) {
+    const uint64_t c = w0 + (uint32_t)lane / share;
+    uint32_t he0 = 0;
+    tl[0] = tl[1] = 0;
+    if (c < nc) {
+      tl[0] = s.ctb[0][c * d.r];
+      tl[1] = s.ctb[0][c * d.r + 1];
+      if (!in_bounds(d, tl[0] < d.hse_cap)) tl[0] = 0;
+      if (!in_bounds(d, tl[1] < d.hse_cap)) tl[1] = 0;
+      he0 = s.pool_col[tl[0]];
+    }
+    extend_rows<2>(d, s, tl, he0, c < nc, lane, view, (uint32_t)lane % share, share);
+  }
+}
+
+constexpr int kListThreads = 1024;
+constexpr uint32_t kSmemKeys = 16384;
+
+// Sorts keys[0..P) (P a power of two) by the whole block. A step whose partners lie within one warp's
+// segment of the keys needs only that warp; the block meets once per step above: 15 barriers
+// for 4096 keys instead of 78.
+__device__ void bitonic(unsigned long long* keys, uint32_t P) {
+  constexpr uint32_t kWarps = kListThreads / 32;
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+  const uint32_t seg = P / kWarps >= 64u ? P / kWarps : 64u;   // keys of one warp
+  const uint32_t lo = wid * seg, hi = lo < P ? (lo + seg < P ? lo + seg : P) : lo;
+  auto step = [&](uint32_t i, uint32_t k, uint32_t j) {
+    const uint32_t ixj = i ^ j;
+    if (ixj > i) {
+      const unsigned long long a = keys[i], b = keys[ixj];
+      const bool up = (i & k) == 0;
+      if ((a > b) == up) { keys[i] = b; keys[ixj] = a; }
+    }
+  };
+  for (uint32_t k = 2; k <= P; k <<= 1) {
+    uint32_t j = k >> 1;
+    for (; j >= seg; j >>= 1) {
+      for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) step(i, k, j);
+      __syncthreads();
+    }
+    for (; j > 0; j >>= 1) {
+      for (uint32_t i = lo + lane; i < hi; i += 32) step(i, k, j);
+      __syncwarp();
+    }
+    if (k >= seg) __syncthreads();   // the next k begins with a step across segments
+  }
+  __syncthreads();
+}
+
+// One block: sort the staged (cip << 32 | R_k) keys, keep the last entry of each
+// cip (its largest R_k), and write the list when it fits the caller's capacity. As the last launch of a slot it
+// also moves the clocks of `tick` on (nothing after it reads the stamps of this slot).
+__global__ void __launch_bounds__(kListThreads) k_list(const Dims d, const Scratch s, uint32_t* ips, uint32_t* rk,
+                                                       uint64_t cap, unsigned long long* n_out_dev,
+                                                       const __grid_constant__ TickArgs tick) {
+  pdl_enter();
+  if ((int)threadIdx.x < tick.n) *tick.tm[threadIdx.x] = tm_next(*tick.tm[threadIdx.x]);
   extern __shared__ unsigned long long skeys[];
   __shared__ unsigned int warp_cnt[kListThreads / 32];
   __shared__ unsigned long long running;
@@ -836,7 +1025,8 @@ __global__ void __launch_bounds__(kListThreads) k_list(const Dims d, const Scrat
 
 cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, uint32_t* rk, uint64_t cap,
                                unsigned long long* n_out_dev, int sms, cudaStream_t st, int* launches,
-                               uint32_t view, bool tensor_pairs) {
+                               uint32_t view, bool tensor_pairs, const TickArgs* tick) {
+  if (tick && (tick->n < 0 || tick->n > kMaxBatch)) return cudaErrorInvalidValue;
   // k_list's and k_pairs_tc's dynamic shared memory limits and k_pairs' occupancy, once per device
   constexpr int kDevices = 64;
   static bool attr[kDevices] = {};
@@ -873,7 +1063,14 @@ cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, u
   }
   if (e != cudaSuccess) return e;
   *launches += 1;
-  for (uint32_t i = 2; i < d.r; ++i) {
+  if (s.bucket_off && !(d.flags & SSD_NO_PRUNE)) {
+    e = launch_pdl(k_extend, (unsigned)(sms * 2), kBlock, 0, st, d, s, view);   // two resident blocks per SM (registers)
+    if (e != cudaSuccess) return e;
+    *launches += 1;
+  }
+  // without pruning every level multiplies, and without the bucket index a candidate probes 2^delta columns:
+  // both want a launch per row, spread evenly
+  for (uint32_t i = 2; i < d.r && (!s.bucket_off || (d.flags & SSD_NO_PRUNE)); ++i) {
     // level 1 (pairs) wrote ctb[0]; level i reads ctb[i & 1] and writes ctb[(i + 1) & 1]
     const uint32_t* rctb = s.ctb[i & 1];
     uint32_t* sctb = s.ctb[(i + 1) & 1];
@@ -881,7 +1078,8 @@ cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, u
     if (e != cudaSuccess) return e;
     *launches += 1;
   }
-  e = launch_pdl(k_list, 1, kListThreads, kSmemKeys * sizeof(unsigned long long), st, d, s, ips, rk, cap, n_out_dev);
+  e = launch_pdl(k_list, 1, kListThreads, kSmemKeys * sizeof(unsigned long long), st, d, s, ips, rk, cap, n_out_dev,
+                 tick ? *tick : TickArgs{});
   *launches += 1;
   return e;
 }
