@@ -77,6 +77,8 @@ thread_local char g_cuda_err[256] = "";
 // Guard words before and after each candidate tuple buffer in the debug build.
 constexpr uint64_t kGuardWords = SSD_DEBUG ? 64 : 0;
 constexpr uint32_t kGuard = 0xC0DEC0DEu;
+// The counters and, behind them, the touch lists' entry counts: a slot clears both at once.
+constexpr uint64_t kCounterBytes = sizeof(ssd::DevCounters) + ssd::kMaxChunks * 4;
 
 int cuda_fail(cudaError_t e, const char* where) {
   std::snprintf(g_cuda_err, sizeof(g_cuda_err), "%s: %s (%s)", where, cudaGetErrorName(e), cudaGetErrorString(e));
@@ -286,7 +288,6 @@ void free_ctx(ssd_ctx* c) {
   }
   cudaFree(c->packed);
   cudaFree(c->tl_ent);
-  cudaFree(c->tl_fill);
 
   cudaFree(c->tables);
   cudaFree(c->hot_idx);
@@ -393,9 +394,8 @@ int ssd_create(const ssd_params* p, const uint32_t* tables, int device, ssd_ctx*
       {(void**)&c->ctb_alloc[1], (d.ctb_cap * R + 2 * kGuardWords) * 4},
       {(void**)&c->dbg, SSD_DEBUG ? 4 : 0},
       {(void**)&c->stage, d.out_cap * 8},
-      {(void**)&c->counters, sizeof(ssd::DevCounters)},
+      {(void**)&c->counters, kCounterBytes},
       {(void**)&c->n_out, 8},
-      {(void**)&c->tl_fill, ssd::kMaxChunks * 4},
       {(void**)&c->bucket_off, NB ? R * (NB + 1) * 4 : 0},
       {(void**)&c->bucket_cnt, NB ? R * NB * 4 : 0},
       {(void**)&c->bucket_ent, NB ? R * d.hse_cap * 4 : 0},
@@ -408,6 +408,7 @@ int ssd_create(const ssd_params* p, const uint32_t* tables, int device, ssd_ctx*
       return SSD_ENOMEM;
     }
   }
+  c->tl_fill = reinterpret_cast<uint32_t*>(c->counters + 1);
   for (int i = 0; i < 2; ++i) c->ctb[i] = c->ctb_alloc[i] + kGuardWords;
   d.touch_bits = c->touch_bytes * 8;
   d.dbg = c->dbg;
@@ -868,7 +869,7 @@ static int slot_chunks1(ssd_ctx* ctx, ssd_sketch* router, const uint32_t* pairs,
     }
     ctx->packed_cap = want;
   }
-  SSD_CUDA(cudaMemsetAsync(ctx->counters, 0, sizeof(ssd::DevCounters), st));
+  SSD_CUDA(cudaMemsetAsync(ctx->counters, 0, kCounterBytes, st));
   rc = trace(ctx, ctx->tr_start, st);
   if (rc != SSD_OK) return rc;
   const uint64_t cnt0 = n_se < count ? n_se : count;
@@ -881,7 +882,6 @@ static int slot_chunks1(ssd_ctx* ctx, ssd_sketch* router, const uint32_t* pairs,
   a.view = router->view;
   cudaError_t e;
   if (lists) {
-    SSD_CUDA(cudaMemsetAsync(ctx->tl_fill, 0, ssd::kMaxChunks * 4, st));
     ssd::ListArgs la;
     la.log2_count = 0;
     while ((1ull << la.log2_count) < count) ++la.log2_count;
@@ -990,11 +990,15 @@ int ssd_slot(ssd_ctx* ctx, ssd_sketch* const* routers, const uint32_t* const* d_
 
   DeviceGuard g(ctx->device);
   cudaStream_t st = as_stream(stream);
-  SSD_CUDA(cudaMemsetAsync(ctx->counters, 0, sizeof(ssd::DevCounters), st));
   int rc = trace(ctx, ctx->tr_start, st);
   if (rc != SSD_OK) return rc;
-  SSD_CUDA(cudaEventRecord(ctx->ev_fork, st));
-  SSD_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+  // one chunk has nothing to overlap its touches with: they stay on `st`, without the events
+  const bool fork = n_chunks > 1;
+  const cudaStream_t touching = fork ? ctx->side : st;
+  if (fork) {
+    SSD_CUDA(cudaEventRecord(ctx->ev_fork, st));
+    SSD_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+  }
   ssd::StreamArgs a;
   std::memset(&a, 0, sizeof(a));
   a.n = n;
@@ -1009,18 +1013,21 @@ int ssd_slot(ssd_ctx* ctx, ssd_sketch* const* routers, const uint32_t* const* d_
     const uint64_t se0 = c * count;
     const uint64_t cnt = n_se - se0 < count ? n_se - se0 : count;
     if (c >= 2) SSD_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev_closed[bsel], 0));  // buffer cleared
-    cudaError_t e = ssd::launch_touch(d, ctx->tables, b, ctx->touch[bsel], se0, cnt, (int)tgrid, ctx->tn, ctx->side);
+    cudaError_t e = ssd::launch_touch(d, ctx->tables, b, ctx->touch[bsel], se0, cnt, (int)tgrid, ctx->tn, touching,
+                                      c == 0 ? ctx->counters : nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "touch kernel");
     ctx->launches += 1;
-    SSD_CUDA(cudaEventRecord(ctx->ev_touched[bsel], ctx->side));
-    SSD_CUDA(cudaStreamWaitEvent(st, ctx->ev_touched[bsel], 0));
+    if (fork) {
+      SSD_CUDA(cudaEventRecord(ctx->ev_touched[bsel], ctx->side));
+      SSD_CUDA(cudaStreamWaitEvent(st, ctx->ev_touched[bsel], 0));
+    }
     a.se0 = se0;
     a.se_count = cnt;
     a.touch = reinterpret_cast<uint8_t*>(ctx->touch[bsel]);
     e = ssd::launch_stream(d, ctx->s, a, ssd::kAdvance | ssd::kHot, ctx->sms, ctx->tn, st);
     if (e != cudaSuccess) return cuda_fail(e, "stream kernel");
     ctx->launches += 1;
-    SSD_CUDA(cudaEventRecord(ctx->ev_closed[bsel], st));
+    if (fork) SSD_CUDA(cudaEventRecord(ctx->ev_closed[bsel], st));
   }
   rc = trace(ctx, ctx->tr_pass, st);
   unsigned long long* nd = d_n_out ? reinterpret_cast<unsigned long long*>(d_n_out) : ctx->n_out;

@@ -302,9 +302,11 @@ cudaError_t launch_stream(const Dims& d, const Scratch& s, const StreamArgs& a, 
 
 // ---- touch collection for the fused slot (ssd_scan.cu) ----
 // Algorithm 2 for the estimators [se0, se0 + se_count) only: instead of storing
-// 0 into the recorder, set its bit in `bits` (layout of StreamArgs::touch).
+// 0 into the recorder, set its bit in `bits` (layout of StreamArgs::touch). clear: the counters of a slot
+// that begins with this launch, or nullptr.
 cudaError_t launch_touch(const Dims& d, const uint32_t* tables, const ScanBatch& b, uint32_t* bits, uint64_t se0,
-                         uint64_t se_count, int grid, const Tuning& tn, cudaStream_t st);
+                         uint64_t se_count, int grid, const Tuning& tn, cudaStream_t st,
+                         DevCounters* clear = nullptr);
 
 // ---- device helpers shared by the scan and streaming kernels ----
 // Simple tabulation: four 256-word tables indexed by the bytes of x, XORed.

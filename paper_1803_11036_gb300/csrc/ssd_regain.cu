@@ -897,10 +897,12 @@ __global__ void __launch_bounds__(kBlock) k_extend(const Dims d, const Scratch s
   const int lane = threadIdx.x & 31;
   const unsigned long long avail = s.counters->level[1];
   const uint64_t nc = avail < d.ctb_cap ? avail : d.ctb_cap;
-  // few candidates: several lanes share one (each takes a part of its row-2 bucket), so that all warps have work
+  // several lanes share a candidate (each takes a part of its row-2 bucket): about as many as a bucket has
+  // entries, and with few candidates more, so that all warps have work
   const uint64_t threads = (uint64_t)gridDim.x * blockDim.x;
+  const uint32_t entries = min(s.counters->hot[2], d.hse_cap) >> d.low_bits;   // of a bucket, on average
   uint32_t share = 1;
-  while (share < 32 && nc * share * 2 <= threads) share *= 2;
+  while (share < 32 && (share < entries || nc * share * 2 <= threads)) share *= 2;
   const uint64_t stride = threads / share;
   const uint32_t per_warp = 32 / share;
   uint32_t tl[SSD_MAX_R];

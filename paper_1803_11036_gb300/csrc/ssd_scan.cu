@@ -125,6 +125,13 @@ __global__ void __launch_bounds__(kBlock) k_scan(const Dims d, const uint32_t* _
   }
 }
 
+// Clears the counters of the slot whose first launch this is (only later launches use them): one operation
+// less in the chain of a small slot. Called by block 0 of the launch.
+__device__ __forceinline__ void clear_counters(DevCounters* c) {
+  if (c && threadIdx.x < sizeof(DevCounters) / 4) reinterpret_cast<uint32_t*>(c)[threadIdx.x] = 0;
+}
+static_assert(sizeof(DevCounters) / 4 <= kBlock, "clear_counters");
+
 // The touch kernels walk the vectors warp by warp (vb = the warp's first
 // vector, a multiple of 32 because the grid stride is): every lane of a warp
 // runs the same iterations, as set_touch<1> needs; a lane past the end only
@@ -132,8 +139,9 @@ __global__ void __launch_bounds__(kBlock) k_scan(const Dims d, const uint32_t* _
 template <int U, int CM>
 __global__ void __launch_bounds__(kBlock) k_touch(const Dims d, const uint32_t* __restrict__ tables,
                                                   const __grid_constant__ ScanBatch b, uint32_t* __restrict__ bits,
-                                                  uint64_t se0, uint64_t count) {
+                                                  uint64_t se0, uint64_t count, DevCounters* clear) {
   __shared__ uint32_t sT[2048];
+  if (blockIdx.x == 0) clear_counters(clear);
   for (int i = threadIdx.x; i < 2048; i += blockDim.x) sT[i] = tables[i];
   __syncthreads();
   const uint32_t r0 = (uint32_t)(se0 >> d.q), r1 = (uint32_t)((se0 + count - 1) >> d.q);
@@ -373,8 +381,8 @@ cudaError_t launch_touch_packed(const Dims& d, const uint4* vec, uint64_t nvec, 
 }
 
 cudaError_t launch_touch(const Dims& d, const uint32_t* tables, const ScanBatch& b, uint32_t* bits, uint64_t se0,
-                         uint64_t se_count, int grid, const Tuning& tn, cudaStream_t st) {
-  SSD_TUNED_LAUNCH(k_touch, grid, st, d, tables, b, bits, se0, se_count);
+                         uint64_t se_count, int grid, const Tuning& tn, cudaStream_t st, DevCounters* clear) {
+  SSD_TUNED_LAUNCH(k_touch, grid, st, d, tables, b, bits, se0, se_count, clear);
   return cudaGetLastError();
 }
 #undef SSD_TUNED_LAUNCH

@@ -13,6 +13,8 @@
 // when one of its recorders was set by a touch or reaches distance 65535.
 // Recorders are read once per pass, in 512-byte coalesced warp accesses with
 // streaming cache hints; the touch bits stay in L2.
+#include <atomic>
+
 #include "ssd_internal.cuh"
 
 namespace ssd {
@@ -613,12 +615,21 @@ __global__ void __launch_bounds__(kBlock, 3) k_chunk(const Dims d, const Scratch
   }
 }
 
+// Resident blocks per SM of a streaming kernel: what fits, at most tn.stream_bps when set. The query costs the
+// host more than a launch, so its answer is kept per device and shared memory size (`seen`, one per kernel).
+constexpr int kDevices = 64;
 template <typename K>
-int blocks_per_sm(K kernel, size_t smem, const Tuning& tn) {
-  int b = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kBlock, smem) != cudaSuccess) return 1;
-  if (tn.stream_bps && (int)tn.stream_bps < b) b = (int)tn.stream_bps;
-  return b > 0 ? b : 1;
+int blocks_per_sm(K kernel, size_t smem, const Tuning& tn, std::atomic<uint64_t>* seen) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return 1;
+  const uint64_t known = seen[dev].load(std::memory_order_relaxed);   // smem << 8 | blocks; 0: not asked yet
+  int b = (int)(known & 255u);
+  if (!b || (known >> 8) != smem) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kBlock, smem) != cudaSuccess) return 1;
+    if (b < 1) b = 1;
+    seen[dev].store(((uint64_t)smem << 8) | (uint64_t)b, std::memory_order_relaxed);
+  }
+  return tn.stream_bps && (int)tn.stream_bps < b ? (int)tn.stream_bps : b;
 }
 
 template <bool ONE, bool ADV, bool HOT, bool TOUCH, int R, int I>
@@ -626,7 +637,8 @@ cudaError_t launch_large(const Dims& d, const Scratch& s, const StreamArgs& a, u
                          const Tuning& tn, cudaStream_t st) {
   const size_t smem = HOT ? (size_t)(kBlock / 32) * (d.eta >> 3) : 0;
   const uint64_t need = (count + (kBlock / 32) - 1) / (kBlock / 32);
-  uint64_t grid = (uint64_t)sms * blocks_per_sm(k_stream_large<ONE, ADV, HOT, TOUCH, R, I>, smem, tn);
+  static std::atomic<uint64_t> seen[kDevices];
+  uint64_t grid = (uint64_t)sms * blocks_per_sm(k_stream_large<ONE, ADV, HOT, TOUCH, R, I>, smem, tn, seen);
   if (grid > need) grid = need;
   k_stream_large<ONE, ADV, HOT, TOUCH, R, I><<<(unsigned)grid, kBlock, smem, st>>>(d, s, a);
   return cudaGetLastError();
@@ -655,7 +667,8 @@ cudaError_t launch_variant(const Dims& d, const Scratch& s, const StreamArgs& a,
   }
   const uint64_t n_units = count * d.eta / 256;
   const uint64_t need = (n_units + (kBlock / 32) - 1) / (kBlock / 32);
-  uint64_t grid = (uint64_t)sms * blocks_per_sm(k_stream_small<ONE, ADV, HOT, TOUCH>, 0, tn);
+  static std::atomic<uint64_t> seen[kDevices];
+  uint64_t grid = (uint64_t)sms * blocks_per_sm(k_stream_small<ONE, ADV, HOT, TOUCH>, 0, tn, seen);
   if (grid > need) grid = need;
   k_stream_small<ONE, ADV, HOT, TOUCH><<<(unsigned)grid, kBlock, 0, st>>>(d, s, a);
   return cudaGetLastError();
@@ -742,7 +755,8 @@ cudaError_t launch_chunk_variant(const Dims& d, const Scratch& s, const ChunkArg
                                  cudaStream_t st) {
   const size_t smem = (size_t)(kBlock / 32) * (d.eta >> 3) + (SRC == kSrcRaw ? 2048 * 4 : 0);
   const uint64_t need = (a.count + (kBlock / 32) - 1) / (kBlock / 32);
-  uint64_t grid = (uint64_t)sms * blocks_per_sm(k_chunk<SRC, CM>, smem, tn);
+  static std::atomic<uint64_t> seen[kDevices];
+  uint64_t grid = (uint64_t)sms * blocks_per_sm(k_chunk<SRC, CM>, smem, tn, seen);
   if (grid > need) grid = need;
   // launched as a programmatic dependent of the previous kernel on the stream (see k_chunk)
   cudaLaunchConfig_t cfg = {};
