@@ -415,10 +415,9 @@ cudaError_t launch_touch_packed(const Dims& d, const uint4* vec, uint64_t nvec, 
                                 uint64_t se0, uint64_t se_count, int grid, const Tuning& tn, cudaStream_t st);
 
 // ---- per-chunk touch lists of the fused slot (ssd_scan.cu) ----
-// Algorithm 2 for every pair of the batch, once per slot, sorted by chunk: chunk c covers the
-// estimators [c * count, (c + 1) * count) of every router, and the touch of router j, estimator
-// se, recorder x has the bit ((j * count + se - c * count) << log2_eta) | touch_pos(x) of that
-// chunk's bits.
+// Algorithm 2 for every pair of one router, once per slot, sorted by chunk: chunk c covers the
+// estimators [c * count, (c + 1) * count), and the touch of estimator se, recorder x has the bit
+// ((se - c * count) << log2_eta) | touch_pos(x) of that chunk's bits.
 // Chunk 0's bits are set directly in `touch0`; the bit index of every touch of chunk c >= 1 is
 // appended to list c (ent + (c - 1) * cap, fill[c] entries). A pair adds at most one touch per
 // row, so a list of a chunk inside one row never holds more than the batch's pairs.

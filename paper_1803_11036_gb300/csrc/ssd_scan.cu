@@ -245,109 +245,182 @@ __global__ void __launch_bounds__(kBlock) k_touch_packed(const Dims d, const uin
   }
 }
 
-// Per-chunk touch lists (see ListArgs). Each block owns a contiguous range of
-// the batch's pair vectors and walks it twice: the first walk sets chunk 0's
-// bits and counts the block's touches per chunk (warp-aggregated shared-memory
-// atomics), one global atomic per chunk then reserves the block's run in each
-// list, and the second walk hashes the same pairs again and writes the bit
-// indices into the reserved runs. The range (about 40 KB at full size) is
-// still in L2 for the second walk. Every lane of a warp runs the same
-// iterations (__match_any_sync needs all 32).
-template <int CM>
-__global__ void __launch_bounds__(kBlock) k_lists(const Dims d, const uint32_t* __restrict__ tables,
+// Per-chunk touch lists of one router (see ListArgs). Each block owns a contiguous range of the pair vectors,
+// each of its warps a fixed share. The first walk counts the warp's touches per chunk, one atomic per
+// chunk then reserves the block's run in each list, and the second walk hashes the pairs, sets
+// chunk 0's bits and writes the other bit indices into the reserved runs. Lane c of a warp keeps chunk c's count,
+// then its place in the list: a touch's rank within the warp comes from a ballot, one per chunk of a row
+// (two at the core-link size), so nothing is counted in shared memory (grouping the lanes by chunk
+// with __match_any_sync and shared atomics took 167 us for 6.25 M pairs, this 111 us). Where a chunk holds
+// whole rows every counted pair has one touch in each and the first walk reads nothing (or, for an IP
+// group's view, the pairs alone); with a single chunk there is no list and no first walk. Every lane of a warp
+// runs the same iterations.
+// SUB: the chunks of a row are 2^SUB (0: whole rows per chunk), or any number for -1.
+template <int CM, int SUB>
+__global__ void __launch_bounds__(kBlock, 4) k_lists(const Dims d, const uint32_t* __restrict__ tables,
                                                   const __grid_constant__ ScanBatch b, const ListArgs a) {
+  constexpr int kWarps = kBlock / 32;
   __shared__ uint32_t sT[2048];
-  __shared__ uint32_t s_cnt[kMaxChunks], s_cur[kMaxChunks];
+  __shared__ uint32_t s_cnt[kWarps][kMaxChunks];
   for (int i = threadIdx.x; i < 2048; i += blockDim.x) sT[i] = tables[i];
-  if (threadIdx.x < kMaxChunks) s_cnt[threadIdx.x] = 0;
   __syncthreads();
-  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
   const uint32_t lt = (1u << lane) - 1u;
-  const uint64_t count = 1ull << a.log2_count;
-  const uint64_t total = b.prefix[b.n];
+  // chunk of (row, col): whole rows (row >> row_shift) or 2^sub of them per row (col >> log2_count)
+  constexpr bool rows = SUB == 0;
+  const uint32_t row_shift = rows ? a.log2_count - d.q : 0u, sub = SUB >= 0 ? (uint32_t)SUB : d.q - a.log2_count;
+  const uint32_t in_chunk = (1u << a.log2_count) - 1u;   // estimator within its chunk
+  const uint64_t total = b.prefix[1];
   uint64_t per = (total + gridDim.x - 1) / gridDim.x;
   per = (per + 31) & ~31ull;
   const uint64_t v0 = (uint64_t)blockIdx.x * per;
   const uint64_t v1 = v0 + per < total ? v0 + per : total;
+  const uint32_t view = b.view[0];
+  const bool group = ((view >> 1) & 31u) != 0u;
+  const uint4* const vec = b.vec[0];
 
-  // the touches of one pair (x, y) of router j: chunk 0's set (first walk), the others counted
-  // (first walk) or written (second walk)
-  auto pair = [&](uint32_t x, uint32_t y, uint32_t view, uint64_t jbase, bool live, bool write) {
-    uint32_t cip = 0, oip = 0;
-    const bool in = live && view_pair(view, x, y, cip, oip);
-    uint32_t xr = 0, c0 = 0;
-    if (in) {
-      xr = tab_hash(sT, oip) & (d.eta - 1u);
-      c0 = tab_hash(sT + 1024, cip) & d.col_mask;
+  auto column = [&](uint32_t i, uint32_t cip, uint32_t c0) {
+    const uint32_t sh = i ? (i - 1u) * d.delta + d.sh0 : 32u;
+    return ((sh < 32u ? (cip >> sh) : 0u) ^ c0) & d.col_mask;
+  };
+  // f(x, y, live) for every pair of the warp's share, in the same order each time
+  auto walk = [&](auto f) {
+    constexpr int U = 2;   // vectors in flight
+    for (uint64_t vb = v0 + wid * 32; vb < v1; vb += U * kBlock) {
+      uint4 w[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        w[u] = vb + u * kBlock + lane < v1 ? __ldcg(vec + vb + u * kBlock + lane) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (vb + u * kBlock >= v1) break;   // warp-uniform
+        const bool live = vb + u * kBlock + lane < v1;
+        f(w[u].x, w[u].y, live);
+        f(w[u].z, w[u].w, live);
+      }
     }
+    if (blockIdx.x == 0 && wid == 0) {   // the packets outside the 16-byte body
+      const uint32_t* e = lane < 2u ? b.edge[lane] : nullptr;
+      f(e ? e[0] : 0u, e ? e[1] : 0u, e != nullptr);
+    }
+  };
+
+  uint32_t mine = 0;   // lane c: this warp's touches of chunk c, then its next place in the list
+  if (a.n_chunks > 1) {
+    if (rows) {
+      uint32_t pairs = 0;
+      if (group) {
+        walk([&](uint32_t x, uint32_t y, bool live) {
+          uint32_t cip, oip;
+          const bool in = view_pair(view, x, y, cip, oip) && live;
+          pairs += __popc(__ballot_sync(0xFFFFFFFFu, in));
+        });
+      } else {
+        for (uint64_t vb = v0 + wid * 32; vb < v1; vb += kBlock)
+          pairs += 2u * (uint32_t)(v1 - vb < 32u ? v1 - vb : 32u);
+        if (blockIdx.x == 0 && wid == 0) pairs += (b.edge[0] != nullptr) + (b.edge[1] != nullptr);
+      }
+      for (uint32_t i = 0; i < d.r; ++i) mine += (i >> row_shift) == lane ? pairs : 0u;
+    } else {
+      walk([&](uint32_t x, uint32_t y, bool live) {
+        uint32_t cip, oip;
+        const bool in = view_pair(view, x, y, cip, oip) && live;
+        const uint32_t c0 = tab_hash(sT + 1024, cip) & d.col_mask;
+        const uint32_t n_in = __popc(__ballot_sync(0xFFFFFFFFu, in));
+#pragma unroll
+        for (uint32_t i = 0; i < SSD_MAX_R; ++i) {
+          if (i < d.r) {
+            const uint32_t c = column(i, cip, c0) >> a.log2_count;
+            if (SUB == 1) {
+              const uint32_t n1 = __popc(__ballot_sync(0xFFFFFFFFu, in && c));
+              mine += lane == 2u * i ? n_in - n1 : lane == 2u * i + 1u ? n1 : 0u;
+            } else {
+              for (uint32_t k = 0; k < (1u << sub); ++k) {
+                const uint32_t n = __popc(__ballot_sync(0xFFFFFFFFu, in && c == k));
+                mine += lane == (i << sub) + k ? n : 0u;
+              }
+            }
+          }
+        }
+      });
+    }
+    s_cnt[wid][lane] = mine;
+    __syncthreads();
+    if (threadIdx.x < kMaxChunks) {   // chunk lane: the block's run, and each warp's part of it
+      uint32_t sum = 0, n[kWarps];
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        n[w] = s_cnt[w][lane];
+        sum += n[w];
+      }
+      uint32_t at = lane >= 1 && lane < a.n_chunks && sum ? atomicAdd(&a.fill[lane], sum) : 0u;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        s_cnt[w][lane] = at;
+        at += n[w];
+      }
+    }
+    __syncthreads();
+    mine = s_cnt[wid][lane];
+  }
+  walk([&](uint32_t x, uint32_t y, bool live) {
+    uint32_t cip, oip;
+    const bool in = view_pair(view, x, y, cip, oip) && live;
+    const uint32_t c0 = tab_hash(sT + 1024, cip) & d.col_mask;
+    const uint32_t pos = touch_pos(d, tab_hash(sT, oip) & (d.eta - 1u));
+    const uint32_t m_in = __ballot_sync(0xFFFFFFFFu, in), n_in = __popc(m_in), r_in = __popc(m_in & lt);
 #pragma unroll
     for (uint32_t i = 0; i < SSD_MAX_R; ++i) {
       if (i < d.r) {
-        uint32_t col = c0;
-        if (i) {
-          const uint32_t sh = (i - 1u) * d.delta + d.sh0;
-          col = ((sh < 32u ? (cip >> sh) : 0u) ^ c0) & d.col_mask;
-        }
-        const uint64_t se = ((uint64_t)i << d.q) | col;
-        const uint32_t c = (uint32_t)(se >> a.log2_count);
-        const uint64_t bit = ((jbase + (se & (count - 1))) << d.log2_eta) | touch_pos(d, xr);
-        if (!write) set_touch<CM>(a.touch0, bit, in && c == 0 && in_bounds(d, bit < d.touch_bits));
-        const uint32_t key = (in && c != 0) ? c : 0xFFFFFFFFu;
-        const uint32_t grp = __match_any_sync(0xFFFFFFFFu, key);
-        if (key != 0xFFFFFFFFu) {
-          const uint32_t leader = __ffs(grp) - 1u;
-          if (!write) {
-            if (lane == leader) atomicAdd(&s_cnt[key], (uint32_t)__popc(grp));
-          } else {
-            uint32_t base = 0;
-            if (lane == leader) base = atomicAdd(&s_cur[key], (uint32_t)__popc(grp));
-            base = __shfl_sync(grp, base, leader);
-            const uint64_t pos = (uint64_t)base + __popc(grp & lt);
-            if (pos < a.cap) a.ent[(uint64_t)(key - 1u) * a.cap + pos] = (uint32_t)bit;
-            else atomicOr(&a.counters->status, SSD_STATUS_INTERNAL);
+        const uint32_t col = column(i, cip, c0);
+        const uint32_t c = rows ? i >> row_shift : (i << sub) + (col >> a.log2_count);
+        const uint32_t se = ((i << d.q) | col) & in_chunk;
+        const uint32_t bit = (se << d.log2_eta) | pos;   // (a chunk's bits number at most 2^32)
+        if (rows ? (i >> row_shift) == 0 : i == 0)   // warp-uniform: some lane may be in chunk 0
+          set_touch<CM>(a.touch0, bit, in && c == 0 && in_bounds(d, bit < d.touch_bits));
+        if (a.n_chunks == 1) continue;
+        uint32_t place = __shfl_sync(0xFFFFFFFFu, mine, c & 31u);
+        if (SUB == 0) {
+          place += r_in;
+          mine += lane == c ? n_in : 0u;
+        } else if (SUB == 1) {
+          const uint32_t m1 = __ballot_sync(0xFFFFFFFFu, in && (c & 1u));
+          const uint32_t r1 = __popc(m1 & lt), n1 = __popc(m1);
+          place += (c & 1u) ? r1 : r_in - r1;
+          mine += lane == 2u * i ? n_in - n1 : lane == 2u * i + 1u ? n1 : 0u;
+        } else {
+          for (uint32_t k = 0; k < (1u << sub); ++k) {
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, in && c == (i << sub) + k);
+            if (c == (i << sub) + k) place += __popc(m & lt);
+            mine += lane == (i << sub) + k ? __popc(m) : 0u;
           }
         }
+        if (in && c != 0) {
+          if (place < a.cap) a.ent[(uint64_t)(c - 1u) * a.cap + place] = bit;
+          else atomicOr(&a.counters->status, SSD_STATUS_INTERNAL);
+        }
       }
     }
-  };
-  auto walk = [&](bool write) {
-    for (uint64_t vb = v0 + (threadIdx.x & ~31u); vb < v1; vb += kBlock) {
-      const uint64_t v = vb + lane;
-      const bool live = v < v1;
-      uint4 w = make_uint4(0, 0, 0, 0);
-      uint64_t jb = 0;
-      uint32_t vw = 0;
-      if (live) {
-        const int j = b.n == 1 ? 0 : find_router(b, v);
-        w = write ? __ldcs(b.vec[j] + (v - b.prefix[j])) : __ldcg(b.vec[j] + (v - b.prefix[j]));
-        jb = (uint64_t)j * count;
-        vw = b.view[j];
-      }
-      pair(w.x, w.y, vw, jb, live, write);
-      pair(w.z, w.w, vw, jb, live, write);
-    }
-    if (blockIdx.x == 0 && threadIdx.x < 32) {   // the packets outside the 16-byte bodies
-      const uint32_t* e = lane < 2u * (uint32_t)b.n ? b.edge[lane] : nullptr;
-      const uint32_t j = lane >> 1;
-      pair(e ? e[0] : 0u, e ? e[1] : 0u, e ? b.view[j] : 0u, (uint64_t)j * count, e != nullptr, write);
-    }
-  };
-  walk(false);
-  __syncthreads();
-  if (threadIdx.x >= 1 && threadIdx.x < a.n_chunks)
-    s_cur[threadIdx.x] = s_cnt[threadIdx.x] ? atomicAdd(&a.fill[threadIdx.x], s_cnt[threadIdx.x]) : 0u;
-  __syncthreads();
-  walk(true);
+  });
 }
 
 }  // namespace
 
 cudaError_t launch_lists(const Dims& d, const uint32_t* tables, const ScanBatch& b, const ListArgs& a, int grid,
                          const Tuning& tn, cudaStream_t st) {
-  if (a.n_chunks > kMaxChunks || b.n > 16) return cudaErrorInvalidValue;
-  if (tn.combine == 1) k_lists<1><<<grid, kBlock, 0, st>>>(d, tables, b, a);
-  else if (tn.combine == 2) k_lists<2><<<grid, kBlock, 0, st>>>(d, tables, b, a);
-  else k_lists<0><<<grid, kBlock, 0, st>>>(d, tables, b, a);
+  static_assert(kMaxChunks == 32, "a lane per chunk");
+  if (a.n_chunks > kMaxChunks || b.n != 1) return cudaErrorInvalidValue;
+  const int sub = a.log2_count >= d.q ? 0 : d.q - a.log2_count == 1 ? 1 : -1;
+#define SSD_LISTS(CM)                                                          \
+  do {                                                                         \
+    if (sub == 0) k_lists<CM, 0><<<grid, kBlock, 0, st>>>(d, tables, b, a);    \
+    else if (sub == 1) k_lists<CM, 1><<<grid, kBlock, 0, st>>>(d, tables, b, a); \
+    else k_lists<CM, -1><<<grid, kBlock, 0, st>>>(d, tables, b, a);            \
+  } while (0)
+  if (tn.combine == 1) SSD_LISTS(1);
+  else if (tn.combine == 2) SSD_LISTS(2);
+  else SSD_LISTS(0);
+#undef SSD_LISTS
   return cudaGetLastError();
 }
 
