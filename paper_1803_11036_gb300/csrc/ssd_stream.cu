@@ -11,8 +11,8 @@
 // every router by one slot. The recorders are stamps (ssd_internal.cuh): the
 // advance itself is the clock's tick, so a router's vector is written back only
 // when one of its recorders was set by a touch or reaches distance 65535.
-// Recorders are read once per pass, in 512-byte coalesced warp accesses with
-// streaming cache hints; the touch bits stay in L2.
+// Recorders are read once per pass, in coalesced warp accesses of 512 bytes or more
+// with the default cache policy (see load_group); the touch bits stay in L2.
 #include <atomic>
 
 #include "ssd_internal.cuh"
@@ -91,12 +91,15 @@ __device__ __forceinline__ uint32_t take_touch(uint8_t* p) {
 
 // Recorder vectors it0 .. it0+m-1 (m <= 8, 32 lanes x 8 recorders each) of the
 // estimator at `base`. All loads of a group are issued before any store of it (a
-// store in between could alias the next load and serialise them).
+// store in between could alias the next load and serialise them). Loads of the default policy, not streaming
+// ones: a touched vector is half a sector, and its store has to find the sector still in L2; with the
+// evict-first loads of a stream it had often gone and was fetched again to be merged (the core-link
+// pass took 1.62 ms so, 1.38 ms now; a pass without touches takes the same time either way).
 __device__ __forceinline__ void load_group(const uint4* r0, uint64_t base, uint32_t it0, uint32_t m, int lane,
                                            uint4 (&v)[8]) {
 #pragma unroll
   for (int u = 0; u < 8; ++u)
-    if (u < (int)m) v[u] = __ldcs(r0 + base + (it0 + u) * 32 + lane);
+    if (u < (int)m) v[u] = r0[base + (it0 + u) * 32 + lane];
 }
 
 // kNever into the recorders of v holding the stamp xe. Out of line: a recorder expires once in
@@ -328,7 +331,7 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
               const uint4* const p = reinterpret_cast<const uint4*>(a.routers[n0 + u]) + base + lane;
 #pragma unroll
               for (int i = 0; i < I; ++i)
-                if (I == 1 || it0 + i < iters) v[u][i] = __ldcs(p + (it0 + i) * 32);
+                if (I == 1 || it0 + i < iters) v[u][i] = p[(it0 + i) * 32];
             }
           }
 #pragma unroll
@@ -428,7 +431,7 @@ __global__ void __launch_bounds__(kBlock) k_stream_small(const Dims d, const Scr
   auto one = [&](int n, uint64_t at, uint8_t* t8) {
     const RouterClock rc = sck[n];
     uint4* rp = reinterpret_cast<uint4*>(a.routers[n]);
-    uint4 v = __ldcs(rp + at);
+    uint4 v = rp[at];
     bool dirty = false;
     if (TOUCH) {
       const uint32_t t = take_touch(t8);
