@@ -295,7 +295,7 @@ def step_rooflines(pk, scan_ms, scan_pk, slot_pass, slot_tail, close_pass, close
             "algorithmic_bytes_model": "2 B read per recorder",
             "achieved_gbs": gbs(rec_bytes, cp), "bound": "hbm", "frac": frac(rec_bytes, cp)},
         "regain_tail": {
-            "what": "pair level, row levels, final test and the sorted list (five launches)",
+            "what": "pair level, row levels, final test and the sorted list (three launches)",
             "ms_per_slice": round(statistics.mean(slot_tail), 4),
             "ms_per_slice_after_close_only": round(statistics.mean(close_tail), 4),
             "bound": "latency (a few MB of bitmaps in L2; SMs mostly idle)"},

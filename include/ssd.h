@@ -377,8 +377,9 @@ SSD_API int ssd_reserve(ssd_ctx* ctx, uint64_t max_pairs);
  *       SMs x this many blocks (1..32);
  *   scan_unroll: 16-byte pair vectors one thread loads before hashing them
  *       (items per thread per step: 1, 2, 4 or 8);
- *   merge_group: routers whose recorders one lane loads before it stores any
- *       of them in the multi-router streaming pass (the merge tile: 2, 4 or 8);
+ *   merge_group: 16-byte vectors of the routers' recorders one lane loads before
+ *       it uses any of them in the multi-router streaming pass (the merge tile: 2,
+ *       4 or 8; 8 is two vectors of each of four routers);
  *   combine_touches: how touches that land on one 32-bit word of the touch
  *       bits are combined. 0 = one atomic per touch; 1 = the lanes of a warp
  *       whose bits fall into one word OR them together (__match_any_sync) and
@@ -386,8 +387,8 @@ SSD_API int ssd_reserve(ssd_ctx* ctx, uint64_t max_pairs);
  *       skipped when the bit is already set, which removes the repeats of a
  *       source that sends many packets to few peers;
  *   collect_touches: where the chunk launches of a one-router ssd_slot find the
- *       next chunk's touches. 0 = per-chunk touch lists: one launch hashes every
- *       pair once per slot, sets chunk 0's touch bits and writes the bit index
+ *       next chunk's touches. 0 = per-chunk touch lists: one launch hashes the
+ *       slot's pairs, sets chunk 0's touch bits and writes the bit index
  *       of every other touch into its chunk's list (4 bytes per touch), so each
  *       chunk launch reads only its own touches; 1 = the slot's pairs, hashed
  *       once into (RHFG[0], H1) words, are re-read by every chunk launch;

@@ -95,8 +95,8 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
 
 // Row i's pooled hot estimators bucketed by the low q-delta bits of their column (one block; counting
 // sort: count, exclusive scan, fill). The counters are kept in the `room` words of shared memory at `sm` where
-// they fit (six barriers and no round trip to L2 in between: about 5 us where 8192 counters in global
-// memory took 20), else in global memory. The order inside a bucket is that of the fill's atomics; the levels
+// they fit (no round trip to L2 between the steps; with 8192 counters in global memory this was most of the
+// launch's 62 us), else in global memory. The order inside a bucket is that of the fill's atomics; the levels
 // do not depend on it (the list is sorted at the end).
 __device__ void build_buckets(const Dims& d, const Scratch& s, uint32_t i, uint32_t* sm, uint32_t room) {
   __shared__ uint32_t part[kBlock / 32];
@@ -378,9 +378,10 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
 }
 
 // At most this many pairs are tested one by one: spread over every warp of the grid, a pair costs eight lanes
-// a few loads, and 40 K pairs of 2048-recorder estimators (20 MB of L2 reads) take 6 us, where the few
-// tiles they make keep a few blocks busy for 16 dependent stages and more (20 x 20 pairs: 15 us, 200 x 200:
-// 17 us). Past about 130 K pairs the tiles, which read each bitmap once per tile, are faster.
+// a few loads, where the few tiles they make keep a few blocks busy for eta / 128 dependent stages each. With
+// 2048-recorder estimators the launch (buckets included) takes 5.6 us for 20 x 20 pairs, 15 us for 40 K and
+// 25 us for 171 K; in tiles it took 30, 62 and 56 us. The direct cost grows with the pairs, the tiles' only
+// with their waves (4.9 M pairs: 55 us), and they meet a little past the limit.
 constexpr uint64_t kDirectPairs = 1u << 18;
 __device__ __forceinline__ void pairs_direct(const Dims& d, const Scratch& s, uint32_t n0, uint32_t n1,
                                              uint32_t blocks) {
