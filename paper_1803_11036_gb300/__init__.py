@@ -398,7 +398,8 @@ class Context:
         are copied behind the call's work and waited for together: one round trip instead of four."""
         torch = _torch()
         head = 0
-        if stream is None:
+        quick = stream is None and ips.dtype == rk.dtype == torch.int32 and n_out.dtype == torch.int64
+        if quick:
             if self._pin is None:
                 self._pin = (torch.empty(1, dtype=torch.int64, pin_memory=True),
                              torch.empty((2, self._HEAD), dtype=torch.int32, pin_memory=True))
@@ -411,7 +412,7 @@ class Context:
         s = self.stats(stream)   # waits for the stream
         if s["status"]:
             raise SSDError(SSD_ECAPACITY, f"{what} (status {s['status']})")
-        if stream is None:
+        if quick:
             m = int(pn[0])
             if m <= head:
                 return pl[0, :m].numpy().view(np.uint32).copy(), pl[1, :m].numpy().view(np.uint32).copy()
