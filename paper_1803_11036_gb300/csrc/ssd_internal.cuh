@@ -123,8 +123,6 @@ __device__ __forceinline__ uint4 flip8(uint4 v, uint32_t tm2) {
 struct Clock {
   uint32_t tm2;     // tm, both halves
   uint32_t lo2;     // oldest stamp in the window, both halves
-  uint32_t hi2;     // newest stamp of the window's range starting at lo (tm, or 65534 when the window
-                    // wraps; k - 1 for distances), both halves
   uint32_t klim2;   // length of the window's 16-bit range, both halves
   uint32_t xe2;     // the stamp whose distance reaches 65535 at the advance, both halves
   uint32_t wrap;    // kNever lies in the 16-bit range of the window
@@ -149,7 +147,6 @@ __host__ __device__ __forceinline__ Clock make_clock(uint32_t tm, uint32_t k) {
   const uint32_t xe = tm_next(tm);
   c.tm2 = tm | (tm << 16);
   c.lo2 = lo | (lo << 16);
-  c.hi2 = wrap ? 0xFFFEFFFEu : c.tm2;
   c.klim2 = klim | (klim << 16);
   c.xe2 = xe | (xe << 16);
   c.wrap = wrap ? 1u : 0u;
@@ -160,7 +157,6 @@ __host__ __device__ __forceinline__ Clock distance_clock(uint32_t k) {
   Clock c;
   c.tm2 = 0u;
   c.lo2 = 0u;
-  c.hi2 = (k - 1u) | ((k - 1u) << 16);
   c.klim2 = k | (k << 16);
   c.xe2 = 0xFFFFFFFFu;   // never matched by a stored value that is advanced (no advance on distances)
   c.wrap = 0u;
@@ -231,10 +227,6 @@ __device__ __forceinline__ uint4 touch_mask_entry(uint32_t t) {
 __device__ __forceinline__ uint4 set_masked(uint4 v, uint4 mk, uint32_t tm2) {
   return make_uint4((v.x & ~mk.x) | (tm2 & mk.x), (v.y & ~mk.y) | (tm2 & mk.y), (v.z & ~mk.z) | (tm2 & mk.z),
                     (v.w & ~mk.w) | (tm2 & mk.w));
-}
-// kNever (0xFFFF) in each recorder whose distance reaches 65535 at the advance, 0 elsewhere.
-__device__ __forceinline__ uint4 expire8(uint4 v, const Clock& c) {
-  return make_uint4(__vcmpeq2(v.x, c.xe2), __vcmpeq2(v.y, c.xe2), __vcmpeq2(v.z, c.xe2), __vcmpeq2(v.w, c.xe2));
 }
 // Clocks of a launch: one per sketch, read from device memory (captured work stays valid as the
 // sketches advance).
