@@ -398,7 +398,11 @@ class Context:
         are copied behind the call's work and waited for together: one round trip instead of four."""
         torch = _torch()
         head = 0
-        quick = stream is None and ips.dtype == rk.dtype == torch.int32 and n_out.dtype == torch.int64
+        # staged only from this device's one-dimensional 4-byte lists on its current stream: a copy out of host
+        # buffers would not wait for the call, and other types and shapes are not copied as they are
+        quick = stream is None and all(t.device == self.device and t.dim() == 1 and t.dtype == torch.int32
+                                       for t in (ips, rk)) and \
+            n_out.device == self.device and n_out.shape == (1,) and n_out.dtype == torch.int64
         if quick:
             if self._pin is None:
                 self._pin = (torch.empty(1, dtype=torch.int64, pin_memory=True),
