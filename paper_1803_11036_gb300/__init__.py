@@ -405,8 +405,10 @@ class Context:
             n_out.device == self.device and n_out.shape == (1,) and n_out.dtype == torch.int64
         if quick:
             if self._pin is None:
-                self._pin = (torch.empty(1, dtype=torch.int64, pin_memory=True),
-                             torch.empty((2, self._HEAD), dtype=torch.int32, pin_memory=True))
+                # ordinary host tensors, whatever mode and default device the first call runs under
+                with torch.inference_mode(False):
+                    self._pin = (torch.empty(1, dtype=torch.int64, device="cpu", pin_memory=True),
+                                 torch.empty((2, self._HEAD), dtype=torch.int32, device="cpu", pin_memory=True))
             head = min(cap, self._HEAD)
             pn, pl = self._pin
             pn.copy_(n_out, non_blocking=True)

@@ -1,5 +1,6 @@
 """Lists fetched with sync=True into every kind of output buffer a call takes: pinned host memory that the device
-writes, a length of another shape, two-dimensional lists. The lists are those of the default buffers."""
+writes, a length of another shape, two-dimensional lists; and with the staging made under inference mode or
+another default device. The lists are those of the default buffers."""
 import numpy as np
 import pytest
 
@@ -49,3 +50,24 @@ def test_output_buffers(case, lists, length):
     n_out = (torch.zeros(1, dtype=torch.int64, pin_memory=True) if length == "pinned" else
              torch.zeros({"1 x 1": (1, 1), "scalar": ()}.get(length, (1,)), dtype=torch.int64, device=ctx.device))
     same(slot((*rows, n_out)), ref)
+
+
+def test_first_fetch_under_inference_mode(case):
+    import torch
+    ctx, slot = case
+    with torch.inference_mode():
+        first = slot()
+    second = slot()
+    same(first, want(ctx, slot))
+    same(second, first)
+
+
+def test_fetch_under_a_cuda_default_device(case):
+    import torch
+    ctx, slot = case
+    torch.set_default_device("cuda:0")
+    try:
+        got = slot()
+    finally:
+        torch.set_default_device(None)
+    same(got, want(ctx, slot))
