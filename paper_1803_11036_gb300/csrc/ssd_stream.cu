@@ -39,35 +39,14 @@ __device__ __forceinline__ uint32_t lt8(uint4 v, uint32_t kk) {
 // The clock of router j of a pass: its tm and expiry stamp in both halves (stamp recorders), or
 // tm2 = 0 and `stamps` false when the pass reads distances.
 struct RouterClock {
-  uint32_t tm2, xe2;
+  uint32_t tm2, xe2, neg_xe2;
 };
-
-// Recorders at vector `at` of the n routers merged exactly, router by router: their distances at their
-// own clocks, the elementwise minimum; with ADV the vectors that hold an expiring recorder are
-// written back. The streaming pass calls it for the lanes its fused form cannot decide. Out of line: they
-// are rare.
-template <bool ADV>
-__device__ __noinline__ uint4 merge_exact(uint16_t* const* routers, const RouterClock* sck, int n, uint64_t at) {
-  uint4 mv = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-#pragma unroll 1
-  for (int j = 0; j < n; ++j) {
-    uint4* const p = reinterpret_cast<uint4*>(routers[j]) + at;
-    const uint4 v = __ldcg(p);
-    const RouterClock rc = sck[j];
-    mv = min8(mv, flip8(v, rc.tm2));
-    if (ADV) {
-      const uint4 e = make_uint4(__vcmpeq2(v.x, rc.xe2), __vcmpeq2(v.y, rc.xe2), __vcmpeq2(v.z, rc.xe2),
-                                 __vcmpeq2(v.w, rc.xe2));
-      if (any8(e)) __stcs(p, or8(v, e));
-    }
-  }
-  return mv;
-}
 __device__ __forceinline__ RouterClock router_clock(const uint32_t* tm) {
   RouterClock rc;
   const uint32_t t = read_tm(tm), xe = tm_next(t);
   rc.tm2 = t | (t << 16);
   rc.xe2 = xe | (xe << 16);
+  rc.neg_xe2 = both(0u - xe);
   return rc;
 }
 
@@ -107,6 +86,20 @@ __device__ __forceinline__ void load_group(const uint4* r0, uint64_t base, uint3
 __device__ __noinline__ uint4 expire_vec(uint4 v, uint32_t xe2) {
   return make_uint4(v.x | __vcmpeq2(v.x, xe2), v.y | __vcmpeq2(v.y, xe2), v.z | __vcmpeq2(v.z, xe2),
                     v.w | __vcmpeq2(v.w, xe2));
+}
+
+// The same for a lane's m vectors (from vector `at` on, 32 apart) of each of the n routers, at their own clocks.
+__device__ __noinline__ void expire_routers(uint16_t* const* routers, const RouterClock* sck, int n, uint64_t at,
+                                            uint32_t m) {
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    uint4* const p = reinterpret_cast<uint4*>(routers[j]) + at;
+    const uint32_t xe2 = sck[j].xe2;
+    for (uint32_t i = 0; i < m; ++i) {
+      const uint4 v = __ldcg(p + i * 32);   // the lane's own (touched) vector
+      if (any_eq8(v, xe2)) __stcs(p + i * 32, expire_vec(v, xe2));
+    }
+  }
 }
 
 // The touch bytes of a lane's m vectors (m = 1, 2, 4 or 8; byte u of the result for its u-th
@@ -260,19 +253,85 @@ __device__ __forceinline__ void pool_if_hot(const Dims& d, const Scratch& s, uin
   __syncwarp();
 }
 
+// The estimators of a block's warps over several routers whose clocks differ (sketches whose slot counters were set),
+// merged as distances, four routers' vectors in flight. Out of line and called before anything else, so that
+// the pass over routers of one clock, which is the common one, does not pay for it in registers. Bound by the
+// instructions of flip8: 16 routers close in 1.26 ms, where those of one clock take 0.75.
+template <bool ADV, bool HOT, bool TOUCH>
+__device__ __noinline__ void stream_clocks(const Dims& d, const Scratch& s, const StreamArgs& a, const RouterClock* sck,
+                                           uint8_t* my, uint64_t count) {
+  constexpr int G = 4;
+  const int lane = threadIdx.x & 31;
+  const uint32_t iters = d.eta >> 8, kk = d.k | (d.k << 16);
+  const uint64_t tstride = count * (d.eta >> 3);
+  uint4* const g = reinterpret_cast<uint4*>(a.global);
+  for (uint64_t se = a.se0 + (uint64_t)blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5); se < a.se0 + count;
+       se += (uint64_t)gridDim.x * (kBlock / 32)) {
+    const uint64_t base = (se << d.log2_eta) >> 3;
+    uint8_t* tb = TOUCH ? a.touch + (se - a.se0) * (d.eta >> 3) + lane * iters : nullptr;
+    uint32_t cnt = 0;
+    for (uint32_t it = 0; it < iters; ++it) {
+      const uint64_t at = base + it * 32 + lane;
+      uint4 mv = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);   // distances
+#pragma unroll 1
+      for (int n0 = 0; n0 < a.n; n0 += G) {
+        const int m = a.n - n0 < G ? a.n - n0 : G;
+        uint4 v[G];
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+          if (u < m) v[u] = reinterpret_cast<const uint4*>(a.routers[n0 + u])[at];
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          if (u < m) {
+            const RouterClock rc = sck[n0 + u];
+            bool dirty = false;
+            if (TOUCH) {
+              const uint32_t t = take_touch(tb + (uint64_t)(n0 + u) * tstride + it);
+              if (t) {
+                v[u] = set8(v[u], t, rc.tm2);
+                dirty = true;
+              }
+            }
+            mv = min8(mv, flip8(v[u], rc.tm2));
+            if (ADV && any_eq8(v[u], rc.xe2)) {
+              v[u] = expire_vec(v[u], rc.xe2);
+              dirty = true;
+            }
+            if (dirty) __stcs(reinterpret_cast<uint4*>(a.routers[n0 + u]) + at, v[u]);
+          }
+        }
+      }
+      if (g) __stcs(g + at, flip8(mv, sck[0].tm2));
+      if (HOT) {
+        const uint32_t bits = lt8(mv, kk);
+        cnt += __popc(bits);
+        my[it * 32 + lane] = (uint8_t)bits;
+      }
+    }
+    if (HOT) pool_if_hot(d, s, se, cnt, my, lane);
+  }
+}
+
 // eta >= 256: one warp per estimator, iters = eta/256 steps of 32 lanes x 8 recorders.
 // One router works on its stamps directly (window test, expiry). Several routers are taken R at a time
 // over I steps, R * I vectors per lane loaded before any is used (fewer routers than 8 would
 // leave too few bytes in flight otherwise). When their clocks agree, which sketches
 // that advance together have, a stamp x is compared as p = x - (tm + 1): the newer the stamp the larger p, except
 // that kNever takes the place `never` = 65534 - tm between the stamps up to tm and the stale ones
-// above tm. The merge is then the running maximum of p, and the running minimum finds what that cannot decide: 0, a
-// recorder that expires; and a maximum of `never` with a smaller minimum, where a stale stamp is the
-// newest (only where it matters: a merged sketch is written, or the window wraps).
-// merge_exact takes those lanes, and every lane when the clocks differ. Two instructions per word and
-// router instead of about twelve: 32 routers of 1.25 GiB each went from 4.2 to 7.3 TB/s (10.3 to 5.9 ms), bound by DRAM.
+// above tm. The merge is then the running maximum of p; where that is `never`, the newest stale stamp decides,
+// which is the running maximum of x + 1 less one (kNever is 0 there, and no stamp up to tm is present).
+// The second maximum is kept only where stale stamps count: a merged sketch is written, or the window wraps.
+// Expiring recorders are found by a running minimum of x - xe, 0 for them, with each router's own xe
+// (expire_routers takes those lanes; a recorder expires once in 65535 slots). Routers whose clocks
+// differ are merged as distances. Two or three instructions per word and router instead of about
+// twelve: 32 routers of 1.25 GiB each went from 4.2 to 7.3 TB/s (10.3 to 5.9 ms), bound by DRAM. The time does not depend
+// on the recorders: 8 sparse routers (160 MiB each) close in 0.45 ms whether their clocks have wrapped or
+// not. Lanes where `never` met a stale stamp once reread every router one by one, and the same close
+// took 1.03 ms just past a wrap. Blocks per SM: 3 hold the vectors in flight; with two vectors (tn.group = 2)
+// a pass without window bits fits 5 in its registers (two routers merged in 614 us, at 4 blocks in 655).
 template <bool ONE, bool ADV, bool HOT, bool TOUCH, int R, int I>
-__global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims d, const Scratch s,
+__global__ void __launch_bounds__(kBlock, ONE ? 4 : R * I <= 2 && !HOT ? 5 : 3) k_stream_large(const __grid_constant__ Dims d,
+                                                         const __grid_constant__ Scratch s,
                                                          const __grid_constant__ StreamArgs a) {
   extern __shared__ __align__(16) uint8_t smask[];
   __shared__ RouterClock sck[ONE ? 1 : kMaxBatch];
@@ -289,6 +348,8 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
   const uint32_t tm0 = read_tm(a.tm[0]);
   const Clock c = stamps ? make_clock(tm0, d.k) : distance_clock(d.k);
   if (a.global_tm && blockIdx.x == 0 && threadIdx.x == 0) *a.global_tm = tm0;
+  constexpr bool MERGE = HOT || !ADV;   // (an advance alone has no merged output)
+  constexpr int NL = MERGE ? 1 : 4;       // (beside the maxima there are registers for one)
   bool same = true;   // several routers: the clocks agree
   if (!ONE) {
     for (int j = threadIdx.x; j < a.n; j += blockDim.x) {
@@ -296,6 +357,10 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
       same = same && sck[j].tm2 == c.tm2;
     }
     same = __syncthreads_and(same);
+    if (MERGE && !same) {
+      stream_clocks<ADV, HOT, TOUCH>(d, s, a, sck, my, count);
+      return;
+    }
   }
   if (ONE && TOUCH) {
     for (int j = threadIdx.x; j < 256; j += blockDim.x) stm[j] = touch_mask_entry((uint32_t)j);
@@ -305,6 +370,14 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
   const uint32_t never2 = both(65534u - tm0);
   Clock pc = c;   // the window test on p
   pc.neg_lo2 = both(tm0 + 1u - c.lo2);
+  constexpr uint32_t kOne2 = 0x00010001u;
+  const bool stale = g != nullptr || (HOT && c.wrap);   // stamps above tm count
+  const uint32_t st_p = both(0u - (tm0 + 2u));          // from x + 1 to p
+  // the largest p, or the newest stale stamp's where that is kNever's (x + 1 = 0 there without one: kNever again)
+  auto or_stale = [&](uint32_t h, uint32_t t) {
+    const uint32_t m = __vcmpeq2(h, never2);
+    return (h & ~m) | (__vadd2(t, st_p) & m);
+  };
 
   for (uint64_t se = a.se0 + (uint64_t)blockIdx.x * (kBlock / 32) + wid; se < se_end; se += wstride) {
     const uint64_t base = (se << d.log2_eta) >> 3;  // in 8-recorder units
@@ -315,12 +388,12 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
       cnt = one_router_se<ADV, HOT, TOUCH>(d, r0, g, base, tb, my, lane, c, stm);
     } else {
       for (uint32_t it0 = 0; it0 < iters; it0 += I) {
-        uint4 hi[I], lo[I];   // running maximum and minimum of p over the routers
+        uint4 hi[I], st[I];   // running maxima over the routers: of p, and of x + 1
+        uint32_t least[NL];   // running minima of x - xe of the lane's vectors
 #pragma unroll
-        for (int i = 0; i < I; ++i) {
-          hi[i] = make_uint4(0u, 0u, 0u, 0u);
-          lo[i] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-        }
+        for (int i = 0; i < I; ++i) hi[i] = st[i] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int i = 0; i < NL; ++i) least[i] = 0xFFFFFFFFu;
         // routers in groups of R: the group's loads are issued before any of its stores
         for (int n0 = 0; n0 < a.n; n0 += R) {
           const int m = a.n - n0 < R ? a.n - n0 : R;
@@ -337,6 +410,7 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
 #pragma unroll
           for (int u = 0; u < R; ++u) {
             if (u < m) {
+              const uint32_t neg_xe2 = MERGE ? c.neg_xe2 : sck[n0 + u].neg_xe2;   // (clocks that differ: an advance alone)
 #pragma unroll
               for (int i = 0; i < I; ++i) {
                 if (I > 1 && it0 + i >= iters) continue;
@@ -350,12 +424,19 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
                   }
                 }
                 const uint4 x = v[u][i];
-                if (HOT || g) {
+                if (MERGE) {
                   hi[i] = make_uint4(add_max2(x.x, to_p, hi[i].x), add_max2(x.y, to_p, hi[i].y),
                                      add_max2(x.z, to_p, hi[i].z), add_max2(x.w, to_p, hi[i].w));
+                  if (stale)
+                    st[i] = make_uint4(add_max2(x.x, kOne2, st[i].x), add_max2(x.y, kOne2, st[i].y),
+                                       add_max2(x.z, kOne2, st[i].z), add_max2(x.w, kOne2, st[i].w));
                 }
-                lo[i] = make_uint4(add_min2(x.x, to_p, lo[i].x), add_min2(x.y, to_p, lo[i].y),
-                                   add_min2(x.z, to_p, lo[i].z), add_min2(x.w, to_p, lo[i].w));
+                if (ADV) {
+                  least[0] = add_min2(x.x, neg_xe2, least[0]);
+                  least[1 % NL] = add_min2(x.y, neg_xe2, least[1 % NL]);
+                  least[2 % NL] = add_min2(x.z, neg_xe2, least[2 % NL]);
+                  least[3 % NL] = add_min2(x.w, neg_xe2, least[3 % NL]);
+                }
               }
             }
           }
@@ -364,21 +445,10 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
         for (int i = 0; i < I; ++i) {
           if (I > 1 && it0 + i >= iters) continue;
           const uint64_t at = base + (it0 + i) * 32 + lane;
-          bool exact = !same;
-          // at tm = 65534 kNever is p = 0 and the expiring stamp 0 is p = 1: every lane with a 0 is taken
-          if (ADV) exact = exact || zero_half(umin2(umin2(lo[i].x, lo[i].y), umin2(lo[i].z, lo[i].w)));
-          if (ADV && tm0 == 65534u) exact = true;
-          if ((HOT && c.wrap) || g) {
-            // 1 in a half whose maximum is `never` while its minimum differs
-            auto stale = [&](uint32_t h, uint32_t l) {
-              return umin2(h ^ l, 0x00010001u) & ~umin2(h ^ never2, 0x00010001u);
-            };
-            exact = exact || ((stale(hi[i].x, lo[i].x) | stale(hi[i].y, lo[i].y) | stale(hi[i].z, lo[i].z) |
-                               stale(hi[i].w, lo[i].w)) & 0x00010001u) != 0u;
-          }
-          if (exact) {
-            const uint4 mv = flip8(merge_exact<ADV>(a.routers, sck, a.n, at), c.tm2);   // stamps at clock tm0
-            hi[i] = make_uint4(__vadd2(mv.x, to_p), __vadd2(mv.y, to_p), __vadd2(mv.z, to_p), __vadd2(mv.w, to_p));
+          if (!MERGE) continue;
+          if (stale) {
+            hi[i] = make_uint4(or_stale(hi[i].x, st[i].x), or_stale(hi[i].y, st[i].y), or_stale(hi[i].z, st[i].z),
+                               or_stale(hi[i].w, st[i].w));
           }
           if (g)
             __stcs(g + at, make_uint4(__vadd2(hi[i].x, from_p), __vadd2(hi[i].y, from_p), __vadd2(hi[i].z, from_p),
@@ -399,6 +469,9 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : 3) k_stream_large(const Dims
             my[(it0 + i) * 32 + lane] = (uint8_t)bits;
           }
         }
+        // (here, where nothing of the merge is live any more: the call would spill it)
+        if (ADV && zero_half(umin2(umin2(least[0], least[1 % NL]), umin2(least[2 % NL], least[3 % NL]))))
+          expire_routers(a.routers, sck, a.n, base + it0 * 32 + lane, iters - it0 < I ? iters - it0 : I);
       }
     }
     if (HOT) pool_if_hot(d, s, se, cnt, my, lane);
