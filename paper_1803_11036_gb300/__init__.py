@@ -400,9 +400,10 @@ class Context:
         head = 0
         # staged only from this device's one-dimensional 4-byte lists on its current stream: a copy out of host
         # buffers would not wait for the call, and other types and shapes are not copied as they are
-        quick = stream is None and all(t.device == self.device and t.dim() == 1 and t.dtype == torch.int32
-                                       for t in (ips, rk)) and \
-            n_out.device == self.device and n_out.shape == (1,) and n_out.dtype == torch.int64
+        dev, word = self.device, torch.int32
+        quick = stream is None and ips.dtype is word and rk.dtype is word and n_out.dtype is torch.int64 and \
+            ips.device == dev and rk.device == dev and n_out.device == dev and \
+            ips.dim() == 1 and rk.dim() == 1 and n_out.dim() == 1
         if quick:
             if self._pin is None:
                 # ordinary host tensors, whatever mode and default device the first call runs under
