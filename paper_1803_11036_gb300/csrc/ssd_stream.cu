@@ -755,11 +755,45 @@ __global__ void k_tick(const __grid_constant__ TickArgs a) {
   if ((int)threadIdx.x < a.n) *a.tm[threadIdx.x] = tm_next(*a.tm[threadIdx.x]);
 }
 
-// dst = flip(src) at one clock; the clock is also stored at tm_out (by one thread). Where both ends reach
-// a 16-byte boundary at the same recorder the body goes in 16-byte vectors, four per thread in flight,
-// and the recorders before and after it one by one; else (an odd `first` against an aligned
-// destination) all of them one by one. Bound by DRAM: a 1.25 GiB RSEA took 1.16 ms one recorder per
-// thread and step (2.3 TB/s read and written), 0.44 ms so.
+// The 16 bytes from byte sh (even, below 16, the same for all lanes) of two consecutive vectors.
+__device__ __forceinline__ uint4 take16(uint4 a, uint4 b, uint32_t sh) {
+  uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  if (sh & 8u) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
+  }
+  if (sh & 4u) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
+  }
+  if (sh & 2u) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], 16);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// The vectors of a flip, four per thread in flight. SHIFT: the source's begin at byte sh of the aligned ones.
+template <bool SHIFT>
+__device__ __forceinline__ void flip_vectors(const uint4* __restrict__ sv, uint4* __restrict__ dv, uint64_t nvec,
+                                             uint32_t sh, uint32_t tm2, uint64_t tid, uint64_t stride) {
+  auto load = [&](uint64_t v) { return SHIFT ? take16(__ldg(sv + v), __ldg(sv + v + 1), sh) : __ldcs(sv + v); };
+  uint64_t v = tid;
+  for (; v + 3 * stride < nvec; v += 4 * stride) {
+    uint4 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = load(v + u * stride);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) __stcs(dv + v + u * stride, flip8(x[u], tm2));
+  }
+  for (; v < nvec; v += stride) __stcs(dv + v, flip8(load(v), tm2));
+}
+
+// dst = flip(src) at one clock; the clock is also stored at tm_out (by one thread). The body goes in 16-byte
+// vectors from the destination's first 16-byte boundary on, and the recorders before and after it
+// one by one. A source that does not reach a boundary at the same recorder (an odd `first` against an aligned
+// destination) is read in its own aligned vectors, two per vector written (the second from L1), all of
+// them inside the source. Bound by DRAM: a 1.25 GiB RSEA took 1.16 ms one recorder per
+// thread and step (2.3 TB/s read and written), 0.44 ms so, 0.47 ms when the ends differ.
 __global__ void __launch_bounds__(kBlock) k_flip(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst,
                                                  uint64_t count, const uint32_t* tm_in, uint32_t tm_val,
                                                  uint32_t* tm_out) {
@@ -769,21 +803,16 @@ __global__ void __launch_bounds__(kBlock) k_flip(const uint16_t* __restrict__ sr
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   uint64_t head = ((16u - (uint32_t)(reinterpret_cast<uintptr_t>(dst) & 15u)) & 15u) >> 1;   // to dst's boundary
+  const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(src + head) & 15u);
+  if (2 * head < sh) head += 8;   // the first aligned source vector begins sh bytes before the body
   if (head > count) head = count;
-  const uint64_t nvec = (reinterpret_cast<uintptr_t>(src + head) & 15u) ? 0 : (count - head) >> 3;
-  const uint4* const sv = reinterpret_cast<const uint4*>(src + head);
+  uint64_t nvec = (count - head + (sh >> 1)) >> 3;
+  if (sh) nvec = nvec ? nvec - 1 : 0;   // vector v is read from the source's aligned vectors v and v + 1
   uint4* const dv = reinterpret_cast<uint4*>(dst + head);
-  uint64_t v = tid;
-  for (; v + 3 * stride < nvec; v += 4 * stride) {
-    uint4 x[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) x[u] = __ldcs(sv + v + u * stride);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) __stcs(dv + v + u * stride, flip8(x[u], tm2));
-  }
-  for (; v < nvec; v += stride) __stcs(dv + v, flip8(__ldcs(sv + v), tm2));
+  if (sh) flip_vectors<true>(reinterpret_cast<const uint4*>(src + head - (sh >> 1)), dv, nvec, sh, tm2, tid, stride);
+  else flip_vectors<false>(reinterpret_cast<const uint4*>(src + head), dv, nvec, 0u, tm2, tid, stride);
   // what the vectors leave out: the head, and everything from `after` on
-  const uint64_t after = nvec ? head + (nvec << 3) : head;
+  const uint64_t after = head + (nvec << 3);
   for (uint64_t i = tid; i < head; i += stride) dst[i] = (uint16_t)flip2(src[i], tm2);
   for (uint64_t i = after + tid; i < count; i += stride) dst[i] = (uint16_t)flip2(src[i], tm2);
 }
