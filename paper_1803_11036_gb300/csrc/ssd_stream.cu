@@ -504,7 +504,9 @@ __global__ void __launch_bounds__(kBlock) k_stream_small(const Dims d, const Scr
   auto one = [&](int n, uint64_t at, uint8_t* t8) {
     const RouterClock rc = sck[n];
     uint4* rp = reinterpret_cast<uint4*>(a.routers[n]);
-    uint4 v = rp[at];
+    // (touched vectors want the default policy, see load_group; without touches 16 routers merge in 267 us by
+    // streaming loads, 290 by default ones)
+    uint4 v = TOUCH ? rp[at] : __ldcs(rp + at);
     bool dirty = false;
     if (TOUCH) {
       const uint32_t t = take_touch(t8);
