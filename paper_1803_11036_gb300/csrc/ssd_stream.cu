@@ -732,14 +732,19 @@ cudaError_t launch_variant(const Dims& d, const Scratch& s, const StreamArgs& a,
     } else {
       // tn.group vectors per lane in flight. Several consecutive ones of fewer routers where an
       // estimator has them: 4 x 2 reads 1 KB of a router at a time, and 16 and 32 routers then stream at
-      // 7.3 TB/s where 8 x 1 (512 B) reaches 6.0
+      // 7.3 TB/s where 8 x 1 (512 B) reaches 6.0. Where 4 x 2 or 8 x 1 loads more routers than there are,
+      // the smaller form leaves registers for more blocks: 2 routers of eta 2048 close with window bits in 448 us by
+      // 2 x 2 (472 by 4 x 2, 481 by 2 x 4, which spills there), advance in 372 us by 2 x 4 (398 by 4 x 2); at
+      // eta 256 2, 3 and 4 routers merge in 183, 212 and 252 us by 4 x 1 (210, 238 and 270 by 8 x 1).
       if (tn.group == 2) return launch_large<false, ADV, HOT, TOUCH, 2, 1>(d, s, a, count, sms, tn, st);
       if (tn.group == 4) {
         if (d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 2, 2>(d, s, a, count, sms, tn, st);
         return launch_large<false, ADV, HOT, TOUCH, 4, 1>(d, s, a, count, sms, tn, st);
       }
-      if (a.n == 2 && d.eta >= 1024) return launch_large<false, ADV, HOT, TOUCH, 2, 4>(d, s, a, count, sms, tn, st);
+      if (a.n == 2 && HOT && d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 2, 2>(d, s, a, count, sms, tn, st);
+      if (a.n == 2 && !HOT && d.eta >= 1024) return launch_large<false, ADV, HOT, TOUCH, 2, 4>(d, s, a, count, sms, tn, st);
       if (d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 4, 2>(d, s, a, count, sms, tn, st);
+      if (a.n <= 4) return launch_large<false, ADV, HOT, TOUCH, 4, 1>(d, s, a, count, sms, tn, st);
       return launch_large<false, ADV, HOT, TOUCH, 8, 1>(d, s, a, count, sms, tn, st);
     }
   }
