@@ -844,85 +844,137 @@ __global__ void __launch_bounds__(kBlock) k_level(const Dims d, const Scratch s,
   }
 }
 
-// The bucket of row-i hot estimators a tuple (rows 0..i-1) can extend to, as a range of bucket_ent.
-__device__ __forceinline__ uint2 extensions(const Dims& d, const Scratch& s, uint32_t i, uint32_t he0,
-                                            const uint32_t (&tl)[SSD_MAX_R]) {
-  uint32_t tp = 0;
-#pragma unroll
-  for (uint32_t j = 0; j < SSD_MAX_R; ++j)
-    if (j == i - 1) tp = tl[j];
-  const uint32_t hep = s.pool_col[(uint64_t)(i - 1) * d.hse_cap + tp];
+// The bucket of row-i hot estimators a tuple can extend to, as a range of bucket_ent: he0 is its row-0 column,
+// `prev` its row i-1 pool index.
+__device__ __forceinline__ uint2 extensions(const Dims& d, const Scratch& s, uint32_t i, uint32_t he0, uint32_t prev) {
+  const uint32_t hep = s.pool_col[(uint64_t)(i - 1) * d.hse_cap + prev];
   const uint32_t low = (he0 ^ ((he0 ^ hep) >> d.delta)) & d.low_mask;
   const uint32_t* off = s.bucket_off + (uint64_t)i * ((1u << d.low_bits) + 1);
   const uint2 be = make_uint2(off[low], off[low + 1]);
   return in_bounds(d, be.x <= be.y && be.y <= d.hse_cap) ? be : make_uint2(0u, 0u);
 }
 
-// The tuples of the warp's `active` lanes (rows 0..I-1) extended through rows I .. r-1, depth first: a
-// kept extension goes on to the next row at once, in its lane, and is counted where the level-by-level
-// form would append it (a count past the candidate buffer's capacity is an overflow there, and
-// here).
-// A lane takes the entries first, first + step, ... of its bucket.
-template <uint32_t I>
-__device__ __forceinline__ void extend_rows(const Dims& d, const Scratch& s, uint32_t (&tl)[SSD_MAX_R], uint32_t he0,
-                                            bool active, int lane, uint32_t view, uint32_t first, uint32_t step) {
-  uint2 be = make_uint2(0u, 0u);
-  if (active) be = extensions(d, s, I, he0, tl);
-  be.x += first;
-  const uint32_t* ent = s.bucket_ent + (uint64_t)I * d.hse_cap;
-  for (; __any_sync(kFull, be.x < be.y); be.x += step) {
-    const uint32_t idx = be.x < be.y ? ent[be.x] : kNone;
-    const uint32_t pc = union_rk(d, s, I, tl, idx, lane);
-    if (I == d.r - 1) {
-      last_hit(d, s, I, tl, idx, pc, view);
-    } else if constexpr (I + 1 < SSD_MAX_R) {
-      bool keep = idx != kNone && pc >= d.thr;
-      const unsigned long long pos = warp_append(keep, &s.counters->level[I]);
-      if (keep && pos >= d.ctb_cap) {
-        atomicOr(&s.counters->status, SSD_STATUS_CTB_OVERFLOW);
-        keep = false;
-      }
-      if (__any_sync(kFull, keep)) {
-        tl[I] = keep ? idx : 0u;
-        extend_rows<I + 1>(d, s, tl, he0, keep, lane, view, 0u, 1u);
-      }
-    }
-  }
-}
-
 // Rows 2 .. r-1 in one launch (pruning on, bucket index there): the pairs that survived are few
 // and their extensions fewer, so a launch per row was three times the latency of one (candidate,
-// bucket, bitmaps, append) and little work. Bound by that latency chain.
-__global__ void __launch_bounds__(kBlock) k_extend(const Dims d, const Scratch s, const uint32_t view) {
+// bucket, bitmaps, append) and little work. A warp keeps the tuples that still have bucket entries to try in
+// queues of its own in shared memory, one per row, and takes 32 entries at a time from the tuples of the
+// deepest queue with kFill of them (nearly full warps, and room for what a step adds); with none, it loads more
+// candidates, and at the end it empties the rows from row 2 on. A kept extension is counted where the
+// level-by-level form would append it (a count past the candidate buffer's capacity is an overflow
+// there, and here). Bound by the latency of that chain with few candidates, by the union tests with many.
+// A lane that extended its own candidates depth first left its warp idle where buckets are long or rows many:
+// with 64 entries a bucket the tail with 36864 tuples of nine pairs took 2.93 ms (0.69 by a launch per row, 0.12
+// now), and with 100 thousand pairs of r = 8 and one entry a bucket 0.63 ms (0.23, 0.18 now).
+constexpr uint32_t kQueue = 48;   // tuples a row's queue holds
+constexpr uint32_t kFill = 16;    // tuples that make a step worth taking; kFill - 1 + 32 fit the queue
+inline uint32_t extend_smem(uint32_t r) { return (kBlock / 32) * (r - 2) * (r + 1) * kQueue * 4; }
+__global__ void __launch_bounds__(kBlock, 2) k_extend(const Dims d, const Scratch s, const uint32_t view) {
   pdl_enter();
+  extern __shared__ uint32_t queues[];
   const int lane = threadIdx.x & 31;
+  const uint32_t below = (1u << lane) - 1u;
+  uint32_t* const q = queues + (threadIdx.x >> 5) * (d.r - 2) * (d.r + 1) * kQueue;
+  // field f of a tuple in row i's queue: its pool indices (rows 0 .. i-1 at 0 ..), the range of entries at r-1 and r
+  auto field = [&](uint32_t i, uint32_t f) { return q + ((i - 2) * (d.r + 1) + f) * kQueue; };
+  uint64_t queued = 0;   // tuples in each row's queue, row i in byte i - 2
+  auto count = [&](uint32_t i) { return (uint32_t)(queued >> (8 * (i - 2))) & 255u; };
+  // queues the lanes' tuples (tl's rows 0 .. i-2, then idx) that have entries in row i
+  auto push = [&](uint32_t i, const uint32_t (&tl)[SSD_MAX_R], uint32_t idx, uint2 be) {
+    const unsigned m = __ballot_sync(kFull, be.x < be.y);
+    const uint32_t t = count(i) + __popc(m & below);
+    if (be.x < be.y) {
+#pragma unroll
+      for (uint32_t j = 0; j < SSD_MAX_R; ++j)
+        if (j + 1 < i) field(i, j)[t] = tl[j];
+      field(i, i - 1)[t] = idx;
+      field(i, d.r - 1)[t] = be.x;
+      field(i, d.r)[t] = be.y;
+    }
+    queued += (uint64_t)__popc(m) << (8 * (i - 2));
+    __syncwarp();
+  };
+
   const unsigned long long avail = s.counters->level[1];
   const uint64_t nc = avail < d.ctb_cap ? avail : d.ctb_cap;
-  // several lanes share a candidate (each takes a part of its row-2 bucket): about as many as a bucket has
-  // entries, and with few candidates more, so that all warps have work
-  const uint64_t threads = (uint64_t)gridDim.x * blockDim.x;
+  // a candidate's bucket is cut into `share` parts: about as many as it has entries, and with few candidates more, so
+  // that all warps have work; the parts go to the warps evenly
+  const uint64_t warps = (uint64_t)gridDim.x * (kBlock / 32);
   const uint32_t entries = min(s.counters->hot[2], d.hse_cap) >> d.low_bits;   // of a bucket, on average
   uint32_t share = 1;
-  while (share < 32 && (share < entries || nc * share * 2 <= threads)) share *= 2;
-  const uint64_t stride = threads / share;
-  const uint32_t per_warp = 32 / share;
-  uint32_t tl[SSD_MAX_R];
-#pragma unroll
-  for (uint32_t j = 0; j < SSD_MAX_R; ++j) tl[j] = 0;
+  while (share < 1024 && (share < entries || (share < 32 && nc * share <= warps * 16))) share *= 2;
+  const uint64_t parts = nc * share;
+  const uint32_t per_warp = parts >= warps * 32 ? 32u : (uint32_t)((parts + warps - 1) / warps);
   // warps in the order of their SMs' first blocks: warp w of block b is the (w * blocks + b)-th
-  const uint64_t warp = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  for (uint64_t w0 = warp * per_warp; w0 < nc; w0 += stride) {
-    const uint64_t c = w0 + (uint32_t)lane / share;
-    uint32_t he0 = 0;
-    tl[0] = tl[1] = 0;
-    if (c < nc) {
-      tl[0] = s.ctb[0][c * d.r];
-      tl[1] = s.ctb[0][c * d.r + 1];
-      if (!in_bounds(d, tl[0] < d.hse_cap)) tl[0] = 0;
-      if (!in_bounds(d, tl[1] < d.hse_cap)) tl[1] = 0;
-      he0 = s.pool_col[tl[0]];
+  uint64_t p0 = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * per_warp;
+  uint32_t tl[SSD_MAX_R];
+  for (;;) {
+    uint32_t i = d.r - 1;
+    while (i >= 2 && count(i) < kFill) --i;
+    if (i < 2) {
+      if (p0 < parts) {   // candidates: row 2's queue takes a tuple per lane
+        const uint64_t p = p0 + lane;
+        uint2 be = make_uint2(0u, 0u);
+#pragma unroll
+        for (uint32_t j = 0; j < SSD_MAX_R; ++j) tl[j] = 0;
+        if (lane < (int)per_warp && p < parts) {
+          const uint64_t c = p / share;
+          const uint32_t part = (uint32_t)(p - c * share);
+          tl[0] = s.ctb[0][c * d.r];
+          tl[1] = s.ctb[0][c * d.r + 1];
+          if (!in_bounds(d, tl[0] < d.hse_cap)) tl[0] = 0;
+          if (!in_bounds(d, tl[1] < d.hse_cap)) tl[1] = 0;
+          be = extensions(d, s, 2, s.pool_col[tl[0]], tl[1]);
+          const uint64_t n = be.y - be.x;
+          be.y = be.x + (uint32_t)(n * (part + 1) / share);
+          be.x += (uint32_t)(n * part / share);
+        }
+        push(2, tl, tl[1], be);
+        p0 += warps * per_warp;
+        continue;
+      }
+      i = 2;
+      while (i < d.r && !count(i)) ++i;
+      if (i == d.r) break;
     }
-    extend_rows<2>(d, s, tl, he0, c < nc, lane, view, (uint32_t)lane % share, share);
+    // up to 32 entries of the queue's last tuples: lane j looks at the j-th from the end, lane l takes the l-th entry
+    const uint32_t n = count(i);
+    const bool mine = (uint32_t)lane < n;
+    const uint32_t t = n - 1 - lane;
+    const uint32_t b = mine ? field(i, d.r - 1)[t] : 0u;
+    const uint32_t rem = mine ? field(i, d.r)[t] - b : 0u;   // 1 or more
+    uint32_t incl = rem;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const uint32_t before = incl - rem;
+    const bool begins = mine && before < 32u;
+    const uint32_t starts = __reduce_or_sync(kFull, begins ? 1u << before : 0u);
+    const uint32_t total = __shfl_sync(kFull, incl, 31);
+    const uint32_t owner = __popc(starts & (below | (1u << lane))) - 1u;   // (lane 0's tuple begins at 0)
+    const uint32_t entry = __shfl_sync(kFull, b, owner) + lane - __shfl_sync(kFull, before, owner);
+    const uint32_t idx = (uint32_t)lane < total ? s.bucket_ent[(uint64_t)i * d.hse_cap + entry] : kNone;
+#pragma unroll
+    for (uint32_t j = 0; j < SSD_MAX_R; ++j) tl[j] = j < i ? field(i, j)[n - 1 - owner] : 0u;
+    __syncwarp();
+    if (begins && incl > 32u) field(i, d.r - 1)[t] = b + 32u - before;   // what is left of the last one
+    queued -= (uint64_t)__popc(__ballot_sync(kFull, mine && incl <= 32u)) << (8 * (i - 2));
+    __syncwarp();
+
+    const uint32_t pc = union_rk(d, s, i, tl, idx, lane);
+    if (i == d.r - 1) {
+      last_hit(d, s, i, tl, idx, pc, view);
+      continue;
+    }
+    bool keep = idx != kNone && pc >= d.thr;
+    const unsigned long long pos = warp_append(keep, &s.counters->level[i]);
+    if (keep && pos >= d.ctb_cap) {
+      atomicOr(&s.counters->status, SSD_STATUS_CTB_OVERFLOW);
+      keep = false;
+    }
+    if (__any_sync(kFull, keep))
+      push(i + 1, tl, idx, keep ? extensions(d, s, i + 1, s.pool_col[tl[0]], idx) : make_uint2(0u, 0u));
   }
 }
 
@@ -1034,6 +1086,7 @@ cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, u
   constexpr int kDevices = 64;
   static bool attr[kDevices] = {};
   static bool tc_attr[kDevices] = {};
+  static bool ext_attr[kDevices] = {};
   static int pair_bps_of[kDevices] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1067,7 +1120,14 @@ cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, u
   if (e != cudaSuccess) return e;
   *launches += 1;
   if (s.bucket_off && !(d.flags & SSD_NO_PRUNE)) {
-    e = launch_pdl(k_extend, (unsigned)(sms * 2), kBlock, 0, st, d, s, view);   // two resident blocks per SM (registers)
+    const uint32_t smem = extend_smem(d.r);   // 27 KB for r = 5
+    if (!ext_attr[dev] && smem > (48u << 10)) {
+      e = cudaFuncSetAttribute(k_extend, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)extend_smem(SSD_MAX_R));
+      if (e != cudaSuccess) return e;
+      ext_attr[dev] = true;
+    }
+    // two resident blocks per SM: a third spills and costs the small regains 2 us more than it gives the large ones
+    e = launch_pdl(k_extend, (unsigned)(sms * 2), kBlock, smem, st, d, s, view);
     if (e != cudaSuccess) return e;
     *launches += 1;
   }
