@@ -953,14 +953,14 @@ def run_ours(args, world, rank, local):
         "default_configuration": default_leg,
         "gbps_at_800B": gbps(value),
         "scan": {"mpps": round(scan_mpps, 2), "gbps_at_800B": gbps(scan_mpps), "ms_per_slice": round(scan_ms, 4),
-                 "note": "ssd_scan alone (recorders written directly; steps.scan_standalone has its roofline); in "
+                 "note": "ssd_scan alone (recorders written directly; step_rooflines.scan_standalone has its roofline); in "
                          "the timed slot the scan's touches go to L2 bits applied by the streaming pass "
-                         "(steps.scan_in_slot)"},
+                         "(step_rooflines.scan_in_slot)"},
         "slot_ms": {"streaming_pass_with_scan": steps["slot_pass"]["ms_per_slice"],
                     "candidates_and_list": steps["regain_tail"]["ms_per_slice"],
                     "total": round(max_ms / args.steps, 4)},
         "reconstruct_ms_per_slice": steps["regain_tail"]["ms_per_slice"],
-        "steps": steps,
+        "step_rooflines": steps,
         "paper_c1": c1,
         "cuda_graph": graph_leg,
         "batched_vs_plain": bvp,
