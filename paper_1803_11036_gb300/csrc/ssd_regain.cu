@@ -982,8 +982,8 @@ constexpr int kListThreads = 1024;
 constexpr uint32_t kSmemKeys = 16384;
 
 // Sorts keys[0..P) (P a power of two) by the whole block. A step whose partners lie within one warp's
-// segment of the keys needs only that warp; the block meets once per step above: 15 barriers
-// for 4096 keys instead of 78.
+// segment of the keys needs only that warp; the block meets once per step above and once per pass that
+// ends in the segments: 21 barriers for 4096 keys instead of 78.
 __device__ void bitonic(unsigned long long* keys, uint32_t P) {
   constexpr uint32_t kWarps = kListThreads / 32;
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
@@ -1007,7 +1007,7 @@ __device__ void bitonic(unsigned long long* keys, uint32_t P) {
       for (uint32_t i = lo + lane; i < hi; i += 32) step(i, k, j);
       __syncwarp();
     }
-    if (k >= seg) __syncthreads();   // the next k begins with a step across segments
+    if (k >= seg && k < P) __syncthreads();   // the next k begins with a step across segments
   }
   __syncthreads();
 }
