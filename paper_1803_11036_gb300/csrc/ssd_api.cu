@@ -382,6 +382,8 @@ int ssd_create(const ssd_params* p, const uint32_t* tables, int device, ssd_ctx*
   const uint64_t NB = d.low_bits <= ssd::kMaxBucketBits ? (1ull << d.low_bits) : 0;  // 0: no bucket index
   c->touch_bytes = p->touch_chunk_bytes ? p->touch_chunk_bytes : (32ull << 20);
   c->touch_bytes = (c->touch_bytes + 255) & ~255ull;
+  // the second candidate buffer: only the launches per row need it (no pruning, or no bucket index)
+  const bool per_row = !NB || (p->flags & SSD_NO_PRUNE);
   struct Alloc { void** ptr; uint64_t bytes; } allocs[] = {
       {(void**)&c->touch[0], c->touch_bytes},
       {(void**)&c->touch[1], c->touch_bytes},
@@ -391,7 +393,7 @@ int ssd_create(const ssd_params* p, const uint32_t* tables, int device, ssd_ctx*
       {(void**)&c->pool_rk, R * d.hse_cap * 4},
       {(void**)&c->pool_bm, R * d.hse_cap * (uint64_t)d.words * 4},
       {(void**)&c->ctb_alloc[0], (d.ctb_cap * R + 2 * kGuardWords) * 4},
-      {(void**)&c->ctb_alloc[1], (d.ctb_cap * R + 2 * kGuardWords) * 4},
+      {(void**)&c->ctb_alloc[1], per_row ? (d.ctb_cap * R + 2 * kGuardWords) * 4 : 0},
       {(void**)&c->dbg, SSD_DEBUG ? 4 : 0},
       {(void**)&c->stage, d.out_cap * 8},
       {(void**)&c->counters, kCounterBytes},
@@ -409,7 +411,7 @@ int ssd_create(const ssd_params* p, const uint32_t* tables, int device, ssd_ctx*
     }
   }
   c->tl_fill = reinterpret_cast<uint32_t*>(c->counters + 1);
-  for (int i = 0; i < 2; ++i) c->ctb[i] = c->ctb_alloc[i] + kGuardWords;
+  for (int i = 0; i < 2; ++i) c->ctb[i] = c->ctb_alloc[i] ? c->ctb_alloc[i] + kGuardWords : nullptr;
   d.touch_bits = c->touch_bytes * 8;
   d.dbg = c->dbg;
   e = cudaMemcpy(c->tables, tables, 2048 * 4, cudaMemcpyHostToDevice);
@@ -419,6 +421,7 @@ int ssd_create(const ssd_params* p, const uint32_t* tables, int device, ssd_ctx*
     uint32_t guard[kGuardWords];
     for (auto& g : guard) g = kGuard;
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+      if (!c->ctb_alloc[i]) continue;
       e = cudaMemcpy(c->ctb_alloc[i], guard, kGuardWords * 4, cudaMemcpyHostToDevice);
       if (e == cudaSuccess)
         e = cudaMemcpy(c->ctb[i] + d.ctb_cap * R, guard, kGuardWords * 4, cudaMemcpyHostToDevice);
@@ -1161,6 +1164,7 @@ int ssd_stats_get(ssd_ctx* ctx, ssd_stats* out, void* stream) {
     uint32_t g[kGuardWords ? kGuardWords : 1];
     const uint64_t words = ctx->d.ctb_cap * ctx->d.r;
     for (int i = 0; i < 2; ++i) {
+      if (!ctx->ctb_alloc[i]) continue;
       for (const uint32_t* at : {ctx->ctb_alloc[i], ctx->ctb[i] + words}) {
         SSD_CUDA(cudaMemcpy(g, at, kGuardWords * 4, cudaMemcpyDeviceToHost));
         for (uint64_t w = 0; w < kGuardWords; ++w)
