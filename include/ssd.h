@@ -379,7 +379,8 @@ SSD_API int ssd_reserve(ssd_ctx* ctx, uint64_t max_pairs);
  *       (items per thread per step: 1, 2, 4 or 8);
  *   merge_group: 16-byte vectors of the routers' recorders one lane loads before
  *       it uses any of them in the multi-router streaming pass (the merge tile: 2,
- *       4 or 8; 8 is two vectors of each of four routers);
+ *       4 or 8; with 8, two vectors of each of four routers, and the smaller tiles
+ *       that suit two to four routers better);
  *   combine_touches: how touches that land on one 32-bit word of the touch
  *       bits are combined. 0 = one atomic per touch; 1 = the lanes of a warp
  *       whose bits fall into one word OR them together (__match_any_sync) and

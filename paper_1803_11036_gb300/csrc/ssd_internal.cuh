@@ -67,8 +67,11 @@ struct Scratch {
   uint32_t* hot_idx;        // [r][2^q] pool index of a hot estimator, kNone otherwise
   uint32_t* pool_col;       // [r][hse_cap] column of each pooled hot estimator
   uint32_t* pool_rk;        // [r][hse_cap] its R_k
-  uint32_t* pool_bm;        // [r][hse_cap][words] bit j = (recorder j < k)
-  uint32_t* ctb[2];         // candidate tuple buffers, tuple stride r (pool indices)
+  uint32_t* pool_bm;        // [r][hse_cap][words] one bit per recorder: inside the window. The order of the bits is free
+                            // within a pass and not the same in all of them (several routers: the eight of
+                            // a byte interleaved by word), so only bitmaps of one pass are compared
+  uint32_t* ctb[2];         // candidate tuple buffers, tuple stride r (pool indices); [1] only where the rows are
+                            // extended by a launch each (no pruning, or no bucket index)
   unsigned long long* stage;  // [out_cap] (cip << 32) | R_k of accepted tuples
   DevCounters* counters;
   // Per row, the pooled hot estimators bucketed by the low q-delta bits of their
@@ -88,7 +91,7 @@ struct Tuning {
   uint32_t stream_bps;   // resident blocks per SM of the streaming kernels (0 = all that fit)
   uint32_t scan_bps;     // scan / touch / pre-hash grid = SMs x scan_bps at most
   uint32_t unroll;       // pair vectors per thread per step: 1, 2, 4, 8
-  uint32_t group;        // routers loaded per lane before storing, multi-router pass: 2, 4, 8
+  uint32_t group;        // 16-byte vectors loaded per lane before any is used, multi-router pass: 2, 4, 8
   uint32_t combine;      // how same-word touch atomics are combined (set_touch's CM)
   uint32_t collect;      // one-router slot: 0 = per-chunk touch lists, 1 = pre-hashed pairs re-read per chunk
   uint32_t pair_level;   // 0 = the pair level on the tensor cores where it applies, 1 = CUDA-core tiles
@@ -126,7 +129,7 @@ struct Clock {
   uint32_t klim2;   // length of the window's 16-bit range, both halves
   uint32_t xe2;     // the stamp whose distance reaches 65535 at the advance, both halves
   uint32_t wrap;    // kNever lies in the 16-bit range of the window
-  // operands of the fused tests (out2, least2), both halves:
+  // operands of the fused tests (out2 and the expiry minimum), both halves:
   uint32_t neg_lo2;    // -lo
   uint32_t top2;       // klim - 1
   uint32_t neg_top2;   // 1 - klim
@@ -286,8 +289,8 @@ struct StreamArgs {
                                        // (j * se_count + e) * eta + x; applied (recorder := 0) and cleared
 };
 // mode bits
-constexpr int kAdvance = 1;   // routers advanced (expired recorders stored as kNever; the clocks are
-                              // moved on by launch_tick after every launch that reads them)
+constexpr int kAdvance = 1;   // routers advanced (expired recorders stored as kNever; the clocks are moved on
+                              // after every launch that reads them: by a slot's last launch, or launch_tick)
 constexpr int kHot = 2;       // count R_k of the merged value and pool the hot estimators
 cudaError_t launch_stream(const Dims& d, const Scratch& s, const StreamArgs& a, int mode, int sms,
                           const Tuning& tn, cudaStream_t st);

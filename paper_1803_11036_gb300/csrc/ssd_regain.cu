@@ -378,10 +378,11 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
 }
 
 // At most this many pairs are tested one by one: spread over every warp of the grid, a pair costs eight lanes
-// a few loads, where the few tiles they make keep a few blocks busy for eta / 128 dependent stages each. With
-// 2048-recorder estimators the launch (buckets included) takes 5.6 us for 20 x 20 pairs, 15 us for 40 K and
-// 25 us for 171 K; in tiles it took 30, 62 and 56 us. The direct cost grows with the pairs, the tiles' only
-// with their waves (4.9 M pairs: 55 us), and they meet a little past the limit.
+// a few loads, where the few tiles they make keep a few blocks busy for eta / 128 dependent stages each. The
+// direct cost grows with the pairs, the tiles' only with their waves. Whole tails at 2^18 and 2^19 pairs none of
+// which survives, direct / tiles in us: eta 512 29 / 42 and 47 / 40, eta 1024 25 / 32 and 40 / 33, eta 2048 32 / 39
+// and 51 / 39, eta 4096 49 / 59 and 85 / 59, eta 8192 58 / 102 and 105 / 102, eta 32768 282 / 383 and 518 / 383;
+// at eta 128 and 256 both take 22 at 2^18. So the crossing lies between the two everywhere.
 constexpr uint64_t kDirectPairs = 1u << 18;
 __device__ __forceinline__ void pairs_direct(const Dims& d, const Scratch& s, uint32_t n0, uint32_t n1,
                                              uint32_t blocks) {
