@@ -398,6 +398,7 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : R * I <= 2 && !HOT ? 5 : 3) 
         for (int n0 = 0; n0 < a.n; n0 += R) {
           const int m = a.n - n0 < R ? a.n - n0 : R;
           uint4 v[R][I];
+          uint32_t tw[R];
 #pragma unroll
           for (int u = 0; u < R; ++u) {
             if (u < m) {
@@ -405,21 +406,22 @@ __global__ void __launch_bounds__(kBlock, ONE ? 4 : R * I <= 2 && !HOT ? 5 : 3) 
 #pragma unroll
               for (int i = 0; i < I; ++i)
                 if (I == 1 || it0 + i < iters) v[u][i] = p[(it0 + i) * 32];
+              // the touch bytes of these I vectors lie side by side (touch_pos)
+              if (TOUCH) tw[u] = (uint32_t)load_touch(tb + (uint64_t)(n0 + u) * tstride + it0, I);
             }
           }
 #pragma unroll
           for (int u = 0; u < R; ++u) {
             if (u < m) {
               const uint32_t neg_xe2 = MERGE ? c.neg_xe2 : sck[n0 + u].neg_xe2;   // (clocks that differ: an advance alone)
+              if (TOUCH) clear_touch(tb + (uint64_t)(n0 + u) * tstride + it0, I, tw[u] != 0u);
 #pragma unroll
               for (int i = 0; i < I; ++i) {
                 if (I > 1 && it0 + i >= iters) continue;
                 if (TOUCH) {
-                  uint8_t* const t8 = tb + (uint64_t)(n0 + u) * tstride + it0 + i;
-                  const uint32_t t = *t8;
+                  const uint32_t t = (tw[u] >> (8 * i)) & 255u;
                   if (t) {
-                    *t8 = 0;
-                    v[u][i] = set8(v[u][i], t, sck[n0 + u].tm2);
+                    v[u][i] = set8(v[u][i], t, c.tm2);
                     __stcs(reinterpret_cast<uint4*>(a.routers[n0 + u]) + base + (it0 + i) * 32 + lane, v[u][i]);
                   }
                 }
@@ -735,16 +737,19 @@ cudaError_t launch_variant(const Dims& d, const Scratch& s, const StreamArgs& a,
       // 7.3 TB/s where 8 x 1 (512 B) reaches 6.0. Where 4 x 2 or 8 x 1 loads more routers than there are,
       // the smaller form leaves registers for more blocks: 2 routers of eta 2048 close with window bits in 448 us by
       // 2 x 2 (472 by 4 x 2, 481 by 2 x 4, which spills there), advance in 372 us by 2 x 4 (398 by 4 x 2); at
-      // eta 256 2, 3 and 4 routers merge in 183, 212 and 252 us by 4 x 1 (210, 238 and 270 by 8 x 1).
+      // eta 256 2, 3 and 4 routers merge in 183, 212 and 252 us by 4 x 1 (210, 238 and 270 by 8 x 1). With touches
+      // the larger forms spill: slots of 4, 8 and 16 routers of eta 2048 take 408, 763 and 1462 us by 2 x 2 (468, 820
+      // and 1450 by 4 x 2), and of 4 routers of eta 256 263 us by 4 x 1 (322 before the touch bytes were loaded
+      // beside the recorders).
       if (tn.group == 2) return launch_large<false, ADV, HOT, TOUCH, 2, 1>(d, s, a, count, sms, tn, st);
       if (tn.group == 4) {
         if (d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 2, 2>(d, s, a, count, sms, tn, st);
         return launch_large<false, ADV, HOT, TOUCH, 4, 1>(d, s, a, count, sms, tn, st);
       }
-      if (a.n == 2 && HOT && d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 2, 2>(d, s, a, count, sms, tn, st);
+      if ((TOUCH || (a.n == 2 && HOT)) && d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 2, 2>(d, s, a, count, sms, tn, st);
       if (a.n == 2 && !HOT && d.eta >= 1024) return launch_large<false, ADV, HOT, TOUCH, 2, 4>(d, s, a, count, sms, tn, st);
       if (d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 4, 2>(d, s, a, count, sms, tn, st);
-      if (a.n <= 4) return launch_large<false, ADV, HOT, TOUCH, 4, 1>(d, s, a, count, sms, tn, st);
+      if (TOUCH || a.n <= 4) return launch_large<false, ADV, HOT, TOUCH, 4, 1>(d, s, a, count, sms, tn, st);
       return launch_large<false, ADV, HOT, TOUCH, 8, 1>(d, s, a, count, sms, tn, st);
     }
   }
