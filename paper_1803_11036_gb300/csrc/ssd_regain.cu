@@ -621,14 +621,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_pairs_tc(const Dims d, const 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols) : "memory");
 }
 
-// Popcount of the AND of the "recorder < k" bitmaps of tuple tl (rows 0..i-1)
-// and row-i estimator idx over words [w0, w0 + n) (n a multiple of 4): all the
-// 16-byte loads of the share are issued before any is used.
-__device__ __forceinline__ uint32_t union_share(const Dims& d, const Scratch& s, uint32_t i,
-                                                const uint32_t (&tl)[SSD_MAX_R], uint32_t idx, uint32_t w0,
-                                                uint32_t n) {
+// Popcount of the AND of the window bitmaps of tuple tl (rows 0..I-1) and row-I estimator idx over words
+// [w0, w0 + n) (n a multiple of 4): all the 16-byte loads of the share are issued before any is used, which takes a row
+// known at compile time (otherwise each row's loads wait for the row before: 10 to 20 % of a regain with many
+// candidates).
+template <uint32_t I>
+__device__ __forceinline__ uint32_t union_share(const Dims& d, const Scratch& s, const uint32_t (&tl)[SSD_MAX_R],
+                                                uint32_t idx, uint32_t w0, uint32_t n) {
   const uint64_t cap = d.hse_cap;
-  const uint32_t* mine = s.pool_bm + ((uint64_t)i * cap + idx) * d.words + w0;
+  const uint32_t* mine = s.pool_bm + ((uint64_t)I * cap + idx) * d.words + w0;
   uint32_t sum = 0;
   for (uint32_t w = 0; w < n; w += 16) {
     uint4 x[4];
@@ -636,15 +637,13 @@ __device__ __forceinline__ uint32_t union_share(const Dims& d, const Scratch& s,
     for (int q = 0; q < 4; ++q) x[q] = w + 4 * q < n ? *reinterpret_cast<const uint4*>(mine + w + 4 * q)
                                                       : make_uint4(0, 0, 0, 0);
 #pragma unroll
-    for (uint32_t j = 0; j < SSD_MAX_R; ++j) {
-      if (j < i) {
-        const uint32_t* row = s.pool_bm + ((uint64_t)j * cap + tl[j]) * d.words + w0 + w;
+    for (uint32_t j = 0; j < I; ++j) {
+      const uint32_t* row = s.pool_bm + ((uint64_t)j * cap + tl[j]) * d.words + w0 + w;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (w + 4 * q < n) {
-            const uint4 y = *reinterpret_cast<const uint4*>(row + 4 * q);
-            x[q].x &= y.x; x[q].y &= y.y; x[q].z &= y.z; x[q].w &= y.w;
-          }
+      for (int q = 0; q < 4; ++q) {
+        if (w + 4 * q < n) {
+          const uint4 y = *reinterpret_cast<const uint4*>(row + 4 * q);
+          x[q].x &= y.x; x[q].y &= y.y; x[q].z &= y.z; x[q].w &= y.w;
         }
       }
     }
@@ -653,12 +652,42 @@ __device__ __forceinline__ uint32_t union_share(const Dims& d, const Scratch& s,
   }
   return sum;
 }
+// The same over the d.words (1 to 8) of a short bitmap, by one lane (the warp taking such hits one after another,
+// a word per lane, made the tail of 5000 hosts of eta 32 7.7 ms, now 0.80).
+template <uint32_t I>
+__device__ __forceinline__ uint32_t union_short(const Dims& d, const Scratch& s, const uint32_t (&tl)[SSD_MAX_R],
+                                                uint32_t idx) {
+  const uint64_t cap = d.hse_cap;
+  uint32_t sum = 0;
+  for (uint32_t w = 0; w < d.words; ++w) {
+    uint32_t x = s.pool_bm[((uint64_t)I * cap + idx) * d.words + w];
+#pragma unroll
+    for (uint32_t j = 0; j < I; ++j) x &= s.pool_bm[((uint64_t)j * cap + tl[j]) * d.words + w];
+    sum += __popc(x);
+  }
+  return sum;
+}
+// The two above for row i of the grid, 2 <= i < R (each row's form is code of its own: R, the rows a kernel is made
+// for, keeps it to those it can meet).
+template <uint32_t R, uint32_t I = 2>
+__device__ __forceinline__ uint32_t union_share_of(uint32_t i, const Dims& d, const Scratch& s,
+                                                   const uint32_t (&tl)[SSD_MAX_R], uint32_t idx, uint32_t w0,
+                                                   uint32_t n) {
+  if constexpr (I + 1 >= R) return union_share<I>(d, s, tl, idx, w0, n);
+  else return i == I ? union_share<I>(d, s, tl, idx, w0, n) : union_share_of<R, I + 1>(i, d, s, tl, idx, w0, n);
+}
+template <uint32_t R, uint32_t I = 2>
+__device__ __forceinline__ uint32_t union_short_of(uint32_t i, const Dims& d, const Scratch& s,
+                                                   const uint32_t (&tl)[SSD_MAX_R], uint32_t idx) {
+  if constexpr (I + 1 >= R) return union_short<I>(d, s, tl, idx);
+  else return i == I ? union_short<I>(d, s, tl, idx) : union_short_of<R, I + 1>(i, d, s, tl, idx);
+}
 
 // R_k of the union for every lane with a hit (idx != kNone; tl its candidate's
 // tuple), computed by the warp together. Every lane of the warp makes the call.
 // With bitmaps of a multiple of 16 words, groups of 4 lanes take up to 8 hits at
-// a time, each lane a quarter of the words; otherwise the whole warp takes the
-// hits one after another.
+// a time, each lane a quarter of the words; shorter ones (1 to 8 words) are each lane's own.
+template <uint32_t R>
 __device__ __forceinline__ uint32_t union_rk(const Dims& d, const Scratch& s, uint32_t i,
                                              const uint32_t (&tl)[SSD_MAX_R], uint32_t idx, int lane) {
   const bool hit = idx != kNone;
@@ -674,9 +703,10 @@ __device__ __forceinline__ uint32_t union_rk(const Dims& d, const Scratch& s, ui
       const int src = busy ? __ffs(mm) - 1 : lane;
       uint32_t tg[SSD_MAX_R];
 #pragma unroll
-      for (uint32_t j = 0; j < SSD_MAX_R; ++j) tg[j] = __shfl_sync(kFull, tl[j], src);
+      for (uint32_t j = 0; j + 1 < R; ++j) tg[j] = __shfl_sync(kFull, tl[j], src);
       const uint32_t ig = __shfl_sync(kFull, idx, src);
-      uint32_t part = busy ? union_share(d, s, i, tg, ig, (lane & 3) * per, per) : 0u;
+      uint32_t part = 0;
+      if (busy) part = union_share_of<R>(i, d, s, tg, ig, (lane & 3) * per, per);
       part += __shfl_xor_sync(kFull, part, 1);
       part += __shfl_xor_sync(kFull, part, 2);
       const uint32_t rank = __popc(m & ((1u << lane) - 1u));
@@ -686,25 +716,7 @@ __device__ __forceinline__ uint32_t union_rk(const Dims& d, const Scratch& s, ui
     }
     return pc;
   }
-  const uint64_t cap = d.hse_cap;
-  while (m) {
-    const int L = __ffs(m) - 1;
-    m &= m - 1;
-    const uint32_t idxL = __shfl_sync(kFull, idx, L);
-    uint32_t tL[SSD_MAX_R];
-#pragma unroll
-    for (uint32_t j = 0; j < SSD_MAX_R; ++j) tL[j] = __shfl_sync(kFull, tl[j], L);
-    uint32_t sum = 0;
-    for (uint32_t w = lane; w < d.words; w += 32) {
-      uint32_t x = s.pool_bm[((uint64_t)i * cap + idxL) * d.words + w];
-#pragma unroll
-      for (uint32_t j = 0; j < SSD_MAX_R; ++j)
-        if (j < i) x &= s.pool_bm[((uint64_t)j * cap + tL[j]) * d.words + w];
-      sum += __popc(x);
-    }
-    sum = __reduce_add_sync(kFull, sum);
-    if (lane == L) pc = sum;
-  }
+  if (hit) pc = union_short_of<R>(i, d, s, tl, idx);
   return pc;
 }
 
@@ -763,7 +775,7 @@ __device__ __forceinline__ void level_hit(const Dims& d, const Scratch& s, uint3
   const bool last = (i == d.r - 1);
   const bool prune = !(d.flags & SSD_NO_PRUNE);
   const bool hit = idx != kNone;
-  const uint32_t pc = (prune || last) ? union_rk(d, s, i, tl, idx, lane) : 0u;
+  const uint32_t pc = (prune || last) ? union_rk<SSD_MAX_R>(d, s, i, tl, idx, lane) : 0u;
   const bool keep = hit && (!prune || pc >= d.thr);
   if (!last) {
     const unsigned long long pos = warp_append(keep, &s.counters->level[i]);
@@ -845,10 +857,9 @@ __global__ void __launch_bounds__(kBlock) k_level(const Dims d, const Scratch s,
   }
 }
 
-// The bucket of row-i hot estimators a tuple can extend to, as a range of bucket_ent: he0 is its row-0 column,
-// `prev` its row i-1 pool index.
-__device__ __forceinline__ uint2 extensions(const Dims& d, const Scratch& s, uint32_t i, uint32_t he0, uint32_t prev) {
-  const uint32_t hep = s.pool_col[(uint64_t)(i - 1) * d.hse_cap + prev];
+// The bucket of row-i hot estimators a tuple can extend to, as a range of bucket_ent; he0 and hep are its columns
+// in the rows 0 and i-1.
+__device__ __forceinline__ uint2 extensions(const Dims& d, const Scratch& s, uint32_t i, uint32_t he0, uint32_t hep) {
   const uint32_t low = (he0 ^ ((he0 ^ hep) >> d.delta)) & d.low_mask;
   const uint32_t* off = s.bucket_off + (uint64_t)i * ((1u << d.low_bits) + 1);
   const uint2 be = make_uint2(off[low], off[low + 1]);
@@ -864,19 +875,21 @@ __device__ __forceinline__ uint2 extensions(const Dims& d, const Scratch& s, uin
 // level-by-level form would append it (a count past the candidate buffer's capacity is an overflow
 // there, and here). Bound by the latency of that chain with few candidates, by the union tests with many.
 // A lane that extended its own candidates depth first left its warp idle where buckets are long or rows many:
-// with 64 entries a bucket the tail with 36864 tuples of nine pairs took 2.93 ms (0.69 by a launch per row, 0.12
-// now), and with 100 thousand pairs of r = 8 and one entry a bucket 0.63 ms (0.23, 0.18 now).
+// with 64 entries a bucket the tail with 36864 tuples of nine pairs took 2.93 ms (0.69 by a launch per row, 0.10
+// now), and with 100 thousand pairs of r = 8 and one entry a bucket 0.63 ms (0.23, 0.14 now). R is d.r: code for the rows
+// that are there only, because a small regain waits for its instructions as well (2 us of a 37 us slot).
 constexpr uint32_t kQueue = 48;   // tuples a row's queue holds
 constexpr uint32_t kFill = 16;    // tuples that make a step worth taking; kFill - 1 + 32 fit the queue
-inline uint32_t extend_smem(uint32_t r) { return (kBlock / 32) * (r - 2) * (r + 1) * kQueue * 4; }
+constexpr uint32_t extend_smem(uint32_t r) { return (kBlock / 32) * (r - 2) * (r + 1) * kQueue * 4; }
+template <uint32_t R>
 __global__ void __launch_bounds__(kBlock, 2) k_extend(const Dims d, const Scratch s, const uint32_t view) {
   pdl_enter();
   extern __shared__ uint32_t queues[];
   const int lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
-  uint32_t* const q = queues + (threadIdx.x >> 5) * (d.r - 2) * (d.r + 1) * kQueue;
+  uint32_t* const q = queues + (threadIdx.x >> 5) * (R - 2) * (R + 1) * kQueue;
   // field f of a tuple in row i's queue: its pool indices (rows 0 .. i-1 at 0 ..), the range of entries at r-1 and r
-  auto field = [&](uint32_t i, uint32_t f) { return q + ((i - 2) * (d.r + 1) + f) * kQueue; };
+  auto field = [&](uint32_t i, uint32_t f) { return q + ((i - 2) * (R + 1) + f) * kQueue; };
   uint64_t queued = 0;   // tuples in each row's queue, row i in byte i - 2
   auto count = [&](uint32_t i) { return (uint32_t)(queued >> (8 * (i - 2))) & 255u; };
   // queues the lanes' tuples (tl's rows 0 .. i-2, then idx) that have entries in row i
@@ -885,11 +898,11 @@ __global__ void __launch_bounds__(kBlock, 2) k_extend(const Dims d, const Scratc
     const uint32_t t = count(i) + __popc(m & below);
     if (be.x < be.y) {
 #pragma unroll
-      for (uint32_t j = 0; j < SSD_MAX_R; ++j)
+      for (uint32_t j = 0; j + 2 < R; ++j)
         if (j + 1 < i) field(i, j)[t] = tl[j];
       field(i, i - 1)[t] = idx;
-      field(i, d.r - 1)[t] = be.x;
-      field(i, d.r)[t] = be.y;
+      field(i, R - 1)[t] = be.x;
+      field(i, R)[t] = be.y;
     }
     queued += (uint64_t)__popc(m) << (8 * (i - 2));
     __syncwarp();
@@ -897,34 +910,34 @@ __global__ void __launch_bounds__(kBlock, 2) k_extend(const Dims d, const Scratc
 
   const unsigned long long avail = s.counters->level[1];
   const uint64_t nc = avail < d.ctb_cap ? avail : d.ctb_cap;
-  // a candidate's bucket is cut into `share` parts: about as many as it has entries, and with few candidates more, so
-  // that all warps have work; the parts go to the warps evenly
+  // a warp takes all entries of its candidates together; with fewer candidates than warps and long buckets, a bucket
+  // is cut into `share` parts, at most one per entry (of a bucket of average length) or warp
   const uint64_t warps = (uint64_t)gridDim.x * (kBlock / 32);
-  const uint32_t entries = min(s.counters->hot[2], d.hse_cap) >> d.low_bits;   // of a bucket, on average
+  const uint32_t entries = min(s.counters->hot[2], d.hse_cap) >> d.low_bits;
   uint32_t share = 1;
-  while (share < 1024 && (share < entries || (share < 32 && nc * share <= warps * 16))) share *= 2;
+  while (share < entries && nc * share * 2 <= warps) share *= 2;
   const uint64_t parts = nc * share;
   const uint32_t per_warp = parts >= warps * 32 ? 32u : (uint32_t)((parts + warps - 1) / warps);
   // warps in the order of their SMs' first blocks: warp w of block b is the (w * blocks + b)-th
   uint64_t p0 = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * per_warp;
   uint32_t tl[SSD_MAX_R];
   for (;;) {
-    uint32_t i = d.r - 1;
+    uint32_t i = R - 1;
     while (i >= 2 && count(i) < kFill) --i;
     if (i < 2) {
       if (p0 < parts) {   // candidates: row 2's queue takes a tuple per lane
         const uint64_t p = p0 + lane;
         uint2 be = make_uint2(0u, 0u);
 #pragma unroll
-        for (uint32_t j = 0; j < SSD_MAX_R; ++j) tl[j] = 0;
+        for (uint32_t j = 0; j + 1 < R; ++j) tl[j] = 0;
         if (lane < (int)per_warp && p < parts) {
           const uint64_t c = p / share;
           const uint32_t part = (uint32_t)(p - c * share);
-          tl[0] = s.ctb[0][c * d.r];
-          tl[1] = s.ctb[0][c * d.r + 1];
+          tl[0] = s.ctb[0][c * R];
+          tl[1] = s.ctb[0][c * R + 1];
           if (!in_bounds(d, tl[0] < d.hse_cap)) tl[0] = 0;
           if (!in_bounds(d, tl[1] < d.hse_cap)) tl[1] = 0;
-          be = extensions(d, s, 2, s.pool_col[tl[0]], tl[1]);
+          be = extensions(d, s, 2, s.pool_col[tl[0]], s.pool_col[d.hse_cap + tl[1]]);
           const uint64_t n = be.y - be.x;
           be.y = be.x + (uint32_t)(n * (part + 1) / share);
           be.x += (uint32_t)(n * part / share);
@@ -934,20 +947,24 @@ __global__ void __launch_bounds__(kBlock, 2) k_extend(const Dims d, const Scratc
         continue;
       }
       i = 2;
-      while (i < d.r && !count(i)) ++i;
-      if (i == d.r) break;
+      while (i < R && !count(i)) ++i;
+      if (i == R) break;
     }
     // up to 32 entries of the queue's last tuples: lane j looks at the j-th from the end, lane l takes the l-th entry
     const uint32_t n = count(i);
     const bool mine = (uint32_t)lane < n;
     const uint32_t t = n - 1 - lane;
-    const uint32_t b = mine ? field(i, d.r - 1)[t] : 0u;
-    const uint32_t rem = mine ? field(i, d.r)[t] - b : 0u;   // 1 or more
+    const uint32_t b = mine ? field(i, R - 1)[t] : 0u;
+    const uint32_t rem = mine ? field(i, R)[t] - b : 0u;   // 1 or more
     uint32_t incl = rem;
+    if (n == 1) {
+      incl = __shfl_sync(kFull, rem, 0);
+    } else {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += y;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
     }
     const uint32_t before = incl - rem;
     const bool begins = mine && before < 32u;
@@ -957,25 +974,33 @@ __global__ void __launch_bounds__(kBlock, 2) k_extend(const Dims d, const Scratc
     const uint32_t entry = __shfl_sync(kFull, b, owner) + lane - __shfl_sync(kFull, before, owner);
     const uint32_t idx = (uint32_t)lane < total ? s.bucket_ent[(uint64_t)i * d.hse_cap + entry] : kNone;
 #pragma unroll
-    for (uint32_t j = 0; j < SSD_MAX_R; ++j) tl[j] = j < i ? field(i, j)[n - 1 - owner] : 0u;
+    for (uint32_t j = 0; j + 1 < R; ++j) tl[j] = j < i ? field(i, j)[n - 1 - owner] : 0u;
     __syncwarp();
-    if (begins && incl > 32u) field(i, d.r - 1)[t] = b + 32u - before;   // what is left of the last one
+    if (begins && incl > 32u) field(i, R - 1)[t] = b + 32u - before;   // what is left of the last one
     queued -= (uint64_t)__popc(__ballot_sync(kFull, mine && incl <= 32u)) << (8 * (i - 2));
     __syncwarp();
 
-    const uint32_t pc = union_rk(d, s, i, tl, idx, lane);
-    if (i == d.r - 1) {
-      last_hit(d, s, i, tl, idx, pc, view);
+    // (the columns that give the next row's range, asked for before the union's loads)
+    uint32_t he0 = 0, hep = 0;
+    if (i < R - 1 && idx != kNone) {
+      he0 = s.pool_col[tl[0]];
+      hep = s.pool_col[(uint64_t)i * d.hse_cap + idx];
+    }
+    const uint32_t pc = union_rk<R>(d, s, i, tl, idx, lane);
+    if (i == R - 1) {
+      last_hit(d, s, R - 1, tl, idx, pc, view);
       continue;
     }
-    bool keep = idx != kNone && pc >= d.thr;
+    const bool keep = idx != kNone && pc >= d.thr;
+    if (!__any_sync(kFull, keep)) continue;
+    // (the count's atomic is under way while that range is read)
     const unsigned long long pos = warp_append(keep, &s.counters->level[i]);
+    uint2 be = keep ? extensions(d, s, i + 1, he0, hep) : make_uint2(0u, 0u);
     if (keep && pos >= d.ctb_cap) {
       atomicOr(&s.counters->status, SSD_STATUS_CTB_OVERFLOW);
-      keep = false;
+      be.y = be.x;
     }
-    if (__any_sync(kFull, keep))
-      push(i + 1, tl, idx, keep ? extensions(d, s, i + 1, s.pool_col[tl[0]], idx) : make_uint2(0u, 0u));
+    push(i + 1, tl, idx, be);
   }
 }
 
@@ -1077,6 +1102,22 @@ __global__ void __launch_bounds__(kListThreads) k_list(const Dims d, const Scrat
   }
 }
 
+constexpr int kDevices = 64;
+
+template <uint32_t R>
+cudaError_t launch_extend(const Dims& d, const Scratch& s, int sms, uint32_t view, cudaStream_t st, int dev) {
+  constexpr uint32_t smem = extend_smem(R);   // 27 KB for R = 5
+  if constexpr (smem > (48u << 10)) {
+    static bool attr[kDevices] = {};
+    if (!attr[dev]) {
+      cudaError_t e = cudaFuncSetAttribute(k_extend<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      attr[dev] = true;
+    }
+  }
+  return launch_pdl(k_extend<R>, (unsigned)(sms * 2), kBlock, smem, st, d, s, view);
+}
+
 }  // namespace
 
 cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, uint32_t* rk, uint64_t cap,
@@ -1084,10 +1125,8 @@ cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, u
                                uint32_t view, bool tensor_pairs, const TickArgs* tick) {
   if (tick && (tick->n < 0 || tick->n > kMaxBatch)) return cudaErrorInvalidValue;
   // k_list's and k_pairs_tc's dynamic shared memory limits and k_pairs' occupancy, once per device
-  constexpr int kDevices = 64;
   static bool attr[kDevices] = {};
   static bool tc_attr[kDevices] = {};
-  static bool ext_attr[kDevices] = {};
   static int pair_bps_of[kDevices] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1121,14 +1160,15 @@ cudaError_t launch_regain_tail(const Dims& d, const Scratch& s, uint32_t* ips, u
   if (e != cudaSuccess) return e;
   *launches += 1;
   if (s.bucket_off && !(d.flags & SSD_NO_PRUNE)) {
-    const uint32_t smem = extend_smem(d.r);   // 27 KB for r = 5
-    if (!ext_attr[dev] && smem > (48u << 10)) {
-      e = cudaFuncSetAttribute(k_extend, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)extend_smem(SSD_MAX_R));
-      if (e != cudaSuccess) return e;
-      ext_attr[dev] = true;
-    }
     // two resident blocks per SM: a third spills and costs the small regains 2 us more than it gives the large ones
-    e = launch_pdl(k_extend, (unsigned)(sms * 2), kBlock, smem, st, d, s, view);
+    switch (d.r) {
+      case 3: e = launch_extend<3>(d, s, sms, view, st, dev); break;
+      case 4: e = launch_extend<4>(d, s, sms, view, st, dev); break;
+      case 5: e = launch_extend<5>(d, s, sms, view, st, dev); break;
+      case 6: e = launch_extend<6>(d, s, sms, view, st, dev); break;
+      case 7: e = launch_extend<7>(d, s, sms, view, st, dev); break;
+      default: e = launch_extend<8>(d, s, sms, view, st, dev);
+    }
     if (e != cudaSuccess) return e;
     *launches += 1;
   }
