@@ -742,15 +742,17 @@ cudaError_t launch_variant(const Dims& d, const Scratch& s, const StreamArgs& a,
       // and 1450 by 4 x 2), and of 4 routers of eta 256 263 us by 4 x 1 (322 before the touch bytes were loaded
       // beside the recorders).
       if (tn.group == 2) return launch_large<false, ADV, HOT, TOUCH, 2, 1>(d, s, a, count, sms, tn, st);
-      if (tn.group == 4) {
+      if (tn.group == 4 || TOUCH) {
         if (d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 2, 2>(d, s, a, count, sms, tn, st);
         return launch_large<false, ADV, HOT, TOUCH, 4, 1>(d, s, a, count, sms, tn, st);
       }
-      if ((TOUCH || (a.n == 2 && HOT)) && d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 2, 2>(d, s, a, count, sms, tn, st);
-      if (a.n == 2 && !HOT && d.eta >= 1024) return launch_large<false, ADV, HOT, TOUCH, 2, 4>(d, s, a, count, sms, tn, st);
-      if (d.eta >= 512) return launch_large<false, ADV, HOT, TOUCH, 4, 2>(d, s, a, count, sms, tn, st);
-      if (TOUCH || a.n <= 4) return launch_large<false, ADV, HOT, TOUCH, 4, 1>(d, s, a, count, sms, tn, st);
-      return launch_large<false, ADV, HOT, TOUCH, 8, 1>(d, s, a, count, sms, tn, st);
+      if constexpr (!TOUCH) {
+        if (a.n == 2 && HOT && d.eta >= 512) return launch_large<false, ADV, HOT, false, 2, 2>(d, s, a, count, sms, tn, st);
+        if (a.n == 2 && !HOT && d.eta >= 1024) return launch_large<false, ADV, HOT, false, 2, 4>(d, s, a, count, sms, tn, st);
+        if (d.eta >= 512) return launch_large<false, ADV, HOT, false, 4, 2>(d, s, a, count, sms, tn, st);
+        if (a.n <= 4) return launch_large<false, ADV, HOT, false, 4, 1>(d, s, a, count, sms, tn, st);
+        return launch_large<false, ADV, HOT, false, 8, 1>(d, s, a, count, sms, tn, st);
+      }
     }
   }
   const uint64_t n_units = count * d.eta / 256;
