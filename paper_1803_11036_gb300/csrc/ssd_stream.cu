@@ -502,13 +502,16 @@ __global__ void __launch_bounds__(kBlock) k_stream_small(const Dims d, const Scr
   for (int j = threadIdx.x; j < (ONE ? 1 : a.n); j += blockDim.x) sck[j] = router_clock(a.tm[j]);
   __syncthreads();
 
+  // Streaming loads in a pass without touches over more than L2 keeps from one slot to the next (129 MB): 16 routers
+  // of eta 64 (2.7 GB) merge in 274 us, 290 by default ones. Touched vectors want the default policy (load_group), and
+  // so do sketches that stay: two routers of eta 32 (84 MB) advance in 39 us, 43 by streaming loads.
+  const bool streaming = !TOUCH && (uint64_t)a.n * count * d.eta * 2 > (96ull << 20);
+
   // router n's vector at `at`: touch applied, written back when it changed; returns its distances
   auto one = [&](int n, uint64_t at, uint8_t* t8) {
     const RouterClock rc = sck[n];
     uint4* rp = reinterpret_cast<uint4*>(a.routers[n]);
-    // (touched vectors want the default policy, see load_group; without touches 16 routers merge in 267 us by
-    // streaming loads, 290 by default ones)
-    uint4 v = TOUCH ? rp[at] : __ldcs(rp + at);
+    uint4 v = streaming ? __ldcs(rp + at) : rp[at];
     bool dirty = false;
     if (TOUCH) {
       const uint32_t t = take_touch(t8);
