@@ -400,9 +400,9 @@ class Context:
         head = 0
         # staged only from this device's one-dimensional 4-byte lists on its current stream: a copy out of host
         # buffers would not wait for the call, and other types and shapes are not copied as they are
-        dev, word = self.device, torch.int32
+        dev, word = self.device.index, torch.int32
         quick = stream is None and ips.dtype is word and rk.dtype is word and n_out.dtype is torch.int64 and \
-            ips.device == dev and rk.device == dev and n_out.device == dev and \
+            ips.get_device() == dev and rk.get_device() == dev and n_out.get_device() == dev and \
             ips.dim() == 1 and rk.dim() == 1 and n_out.dim() == 1
         if quick:
             if self._pin is None:
