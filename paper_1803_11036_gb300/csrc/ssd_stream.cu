@@ -789,10 +789,30 @@ __device__ __forceinline__ uint4 take16(uint4 a, uint4 b, uint32_t sh) {
   }
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
-// The vectors of a flip, four per thread in flight. SHIFT: the source's begin at byte sh of the aligned ones.
+// dst = flip(src) at one clock; the clock is also stored at tm_out (by one thread). The body goes in 16-byte
+// vectors from the destination's first 16-byte boundary on, and the recorders before and after it
+// one by one. A source that does not reach a boundary at the same recorder (an odd `first` against an aligned
+// destination) is read in its own aligned vectors, two per vector written (the second from L1), all of
+// them inside the source. Bound by DRAM: a 1.25 GiB RSEA took 1.16 ms one recorder per
+// thread and step (2.3 TB/s read and written), 0.44 ms so, 0.47 ms when the ends differ.
+// SHIFT: the source begins at another byte of its 16 than the destination (chosen by the host).
 template <bool SHIFT>
-__device__ __forceinline__ void flip_vectors(const uint4* __restrict__ sv, uint4* __restrict__ dv, uint64_t nvec,
-                                             uint32_t sh, uint32_t tm2, uint64_t tid, uint64_t stride) {
+__global__ void __launch_bounds__(kBlock) k_flip(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst,
+                                                 uint64_t count, const uint32_t* tm_in, uint32_t tm_val,
+                                                 uint32_t* tm_out) {
+  const uint32_t tm = tm_in ? *tm_in : tm_val;
+  const uint32_t tm2 = tm | (tm << 16);
+  if (tm_out && blockIdx.x == 0 && threadIdx.x == 0) *tm_out = tm;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  uint64_t head = ((16u - (uint32_t)(reinterpret_cast<uintptr_t>(dst) & 15u)) & 15u) >> 1;   // to dst's boundary
+  const uint32_t sh = SHIFT ? (uint32_t)(reinterpret_cast<uintptr_t>(src + head) & 15u) : 0u;
+  if (SHIFT && 2 * head < sh) head += 8;   // the first aligned source vector begins sh bytes before the body
+  if (head > count) head = count;
+  uint64_t nvec = (count - head + (sh >> 1)) >> 3;
+  if (SHIFT) nvec = nvec ? nvec - 1 : 0;   // vector v is read from the source's aligned vectors v and v + 1
+  const uint4* const sv = reinterpret_cast<const uint4*>(src + head - (sh >> 1));
+  uint4* const dv = reinterpret_cast<uint4*>(dst + head);
   auto load = [&](uint64_t v) { return SHIFT ? take16(__ldg(sv + v), __ldg(sv + v + 1), sh) : __ldcs(sv + v); };
   uint64_t v = tid;
   for (; v + 3 * stride < nvec; v += 4 * stride) {
@@ -803,31 +823,6 @@ __device__ __forceinline__ void flip_vectors(const uint4* __restrict__ sv, uint4
     for (int u = 0; u < 4; ++u) __stcs(dv + v + u * stride, flip8(x[u], tm2));
   }
   for (; v < nvec; v += stride) __stcs(dv + v, flip8(load(v), tm2));
-}
-
-// dst = flip(src) at one clock; the clock is also stored at tm_out (by one thread). The body goes in 16-byte
-// vectors from the destination's first 16-byte boundary on, and the recorders before and after it
-// one by one. A source that does not reach a boundary at the same recorder (an odd `first` against an aligned
-// destination) is read in its own aligned vectors, two per vector written (the second from L1), all of
-// them inside the source. Bound by DRAM: a 1.25 GiB RSEA took 1.16 ms one recorder per
-// thread and step (2.3 TB/s read and written), 0.44 ms so, 0.47 ms when the ends differ.
-__global__ void __launch_bounds__(kBlock) k_flip(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst,
-                                                 uint64_t count, const uint32_t* tm_in, uint32_t tm_val,
-                                                 uint32_t* tm_out) {
-  const uint32_t tm = tm_in ? *tm_in : tm_val;
-  const uint32_t tm2 = tm | (tm << 16);
-  if (tm_out && blockIdx.x == 0 && threadIdx.x == 0) *tm_out = tm;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint64_t head = ((16u - (uint32_t)(reinterpret_cast<uintptr_t>(dst) & 15u)) & 15u) >> 1;   // to dst's boundary
-  const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(src + head) & 15u);
-  if (2 * head < sh) head += 8;   // the first aligned source vector begins sh bytes before the body
-  if (head > count) head = count;
-  uint64_t nvec = (count - head + (sh >> 1)) >> 3;
-  if (sh) nvec = nvec ? nvec - 1 : 0;   // vector v is read from the source's aligned vectors v and v + 1
-  uint4* const dv = reinterpret_cast<uint4*>(dst + head);
-  if (sh) flip_vectors<true>(reinterpret_cast<const uint4*>(src + head - (sh >> 1)), dv, nvec, sh, tm2, tid, stride);
-  else flip_vectors<false>(reinterpret_cast<const uint4*>(src + head), dv, nvec, 0u, tm2, tid, stride);
   // what the vectors leave out: the head, and everything from `after` on
   const uint64_t after = head + (nvec << 3);
   for (uint64_t i = tid; i < head; i += stride) dst[i] = (uint16_t)flip2(src[i], tm2);
@@ -848,7 +843,11 @@ cudaError_t launch_flip(const uint16_t* src, uint16_t* dst, uint64_t count, cons
   uint64_t grid = (count + kBlock - 1) / kBlock;
   if (grid > (uint64_t)sms * 8) grid = (uint64_t)sms * 8;
   if (grid < 1) grid = 1;
-  k_flip<<<(unsigned)grid, kBlock, 0, st>>>(src, dst, count, tm_in, tm_val, tm_out);
+  // the two ends reach a 16-byte boundary at the same recorder, or not
+  if ((reinterpret_cast<uintptr_t>(src) ^ reinterpret_cast<uintptr_t>(dst)) & 15u)
+    k_flip<true><<<(unsigned)grid, kBlock, 0, st>>>(src, dst, count, tm_in, tm_val, tm_out);
+  else
+    k_flip<false><<<(unsigned)grid, kBlock, 0, st>>>(src, dst, count, tm_in, tm_val, tm_out);
   return cudaGetLastError();
 }
 
